@@ -33,17 +33,25 @@ __device__ uint32_t g_u_isb4[256];
 
 namespace {
 
-// Regions A = Te0|Te1, B = Td0|Td1, C = S4|IS4, each row replicated per lane.
+// Regions A = Te0|Te1, B = Td0|Td1, C = S4|IS4, each row replicated per lane:
+// 16 pieces of 16 bytes per row, one 16-byte store per piece and region (the
+// 192 KiB in 1,536 wavefronts; as the bulk kernels' fill, one launch's fixed
+// cost).
 __device__ __forceinline__ void fill_unified(char* smem) {
-    uint32_t* w = reinterpret_cast<uint32_t*>(smem);
-    for (uint32_t i = threadIdx.x; i < 3 * 16384; i += blockDim.x) {
-        uint32_t region = i >> 14, x = (i >> 6) & 255u, half = (i >> 5) & 1u;
-        uint32_t v;
-        if (region == 0) v = g_u_te0[x];
-        else if (region == 1) v = g_u_td0[x];
-        else v = half ? g_u_isb4[x] : g_u_sb4[x];
-        if (region < 2 && half) v = rotl8(v);
-        w[i] = v;
+    uint4* w = reinterpret_cast<uint4*>(smem);
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < 4096; i += blockDim.x) {
+        const uint32_t x = i >> 4;
+        const bool odd = (i & 8u) != 0;
+        uint32_t a = g_u_te0[x], b = g_u_td0[x];
+        const uint32_t c = odd ? g_u_isb4[x] : g_u_sb4[x];
+        if (odd) {
+            a = rotl8(a);
+            b = rotl8(b);
+        }
+        w[i] = make_uint4(a, a, a, a);
+        w[4096 + i] = make_uint4(b, b, b, b);
+        w[8192 + i] = make_uint4(c, c, c, c);
     }
 }
 
