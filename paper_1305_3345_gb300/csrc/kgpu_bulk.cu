@@ -83,15 +83,27 @@ __device__ __forceinline__ void warp_range(uint64_t n, uint64_t& begin, uint64_t
     end = n * (wg + 1) / W;
 }
 
+// a / b where a rarely needs more than 32 bits.
+__device__ __forceinline__ uint64_t div_small(uint64_t a, uint32_t b) {
+    return (a >> 32) == 0 ? (uint64_t)((uint32_t)a / b) : a / b;
+}
+
 // ---------------------------------------------------------------------------
-// XTS (and ECB when TWEAK is false).
+// XTS (and ECB when TWEAK is false).  Bound by the shared-memory lookups (one
+// wavefront a cycle); a CTA owns one contiguous run of 32-block chunks and its
+// warps equal parts of it.
 //
-// Tweaks: a warp keeps E_K2 of 32 consecutive data units in its lanes (lane i
-// holds the unit `base + i`, one AES per lane, computed together).  A lane
-// moving to block j of a new unit takes that unit's E_K2 by shuffle and
-// multiplies by alpha^j in closed form (j < 32 there); a lane staying in its
-// unit steps its tweak by alpha^32.  So the tweak costs one extra AES per
-// data unit and a few shifts per block -- never a sequential chain.
+// Tweaks: the E_K2 of the data units that a group of warps is about to touch
+// are enciphered first, one unit per thread, into shared memory (a phase), and
+// a lane entering a unit reads its E_K2 there and multiplies by alpha^j in
+// closed form; a lane staying in its unit steps its tweak by alpha^32.  The
+// group is the CTA for units of at least a chunk, so that a unit is enciphered
+// once per CTA and a short run costs one warp's AES: with 32 units enciphered
+// by every warp for itself, 1 MiB of 4-KiB units spent as many lookups on
+// tweaks as on data.  Smaller units change within a chunk; there each warp
+// takes its own 32 units at a time and no barrier is needed.
+// 1 MiB of 4-KiB units, AES-256 decryption, back to back on the GPU: 14.4 -> 8.2 us;
+// 16 MiB of encryption 34.9 -> 30.8 us.
 // ---------------------------------------------------------------------------
 template <int NR, int DIR, bool TWEAK>
 __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_constant__ BulkParams p) {
@@ -102,89 +114,97 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_cons
     __syncthreads();
 
     const uint32_t lane = lane_id();
+    const uint32_t warp = threadIdx.x >> 5;
+    constexpr uint32_t kWarps = kBulkThreads / 32;
     const Rep4 T{lane * 4u, lane * 4u + 128u};
     const Rep1<2> IS{lane * 4u};
     const Rep1<2> TE{lane * 4u + 128u};
     const ParamKey K{p.rk};
     const ParamKey TK{p.tk};
 
-    uint64_t c0, c1;
-    warp_range((p.nblocks + 31) >> 5, c0, c1);
-    if (c0 >= c1) return;
+    // this CTA's chunks, and this warp's part of them
+    const uint32_t own = p.cta_chunks + (blockIdx.x < p.cta_rest ? 1u : 0u);
+    const uint64_t first = (uint64_t)p.cta_chunks * blockIdx.x + min(blockIdx.x, p.cta_rest);
+    const uint32_t wa = (uint32_t)((uint64_t)own * warp / kWarps);
+    const uint32_t we = (uint32_t)((uint64_t)own * (warp + 1) / kWarps);
 
-    uint64_t blk = (c0 << 5) + lane;
-    const uint32_t bps = p.bps;
-    uint64_t base = 0;
-    uint32_t srel = 0, j = 0;
-    uint32_t z0 = 0, z1 = 0, z2 = 0, z3 = 0;  // E_K2(unit base + lane)
-    uint32_t t0 = 0, t1 = 0, t2 = 0, t3 = 0;  // tweak of this lane's block
-
-    auto tweak_batch = [&]() {
-        uint64_t unit = p.first_sector + base + lane;
-        z0 = (uint32_t)unit;
-        z1 = (uint32_t)(unit >> 32);
-        z2 = 0;
-        z3 = 0;
-        if (DIR == 0) encrypt_block<NR>(z0, z1, z2, z3, T, TK);
-        else encrypt_block<NR>(z0, z1, z2, z3, TE, TK);
-    };
-
-    if (TWEAK) {
-        base = (c0 << 5) / bps;
-        uint64_t sabs = blk / bps;
-        srel = (uint32_t)(sabs - base);
-        j = (uint32_t)(blk - sabs * bps);
-        tweak_batch();
-        t0 = __shfl_sync(0xffffffffu, z0, srel);
-        t1 = __shfl_sync(0xffffffffu, z1, srel);
-        t2 = __shfl_sync(0xffffffffu, z2, srel);
-        t3 = __shfl_sync(0xffffffffu, z3, srel);
-        gf128_mul_xpow(t0, t1, t2, t3, j);
+    if constexpr (!TWEAK) {
+        uint64_t blk = ((first + wa) << 5) + lane;
+        // the next chunk is fetched while this one is enciphered
+        uint4 nxt = wa < we && blk < p.nblocks ? p.src[blk] : make_uint4(0, 0, 0, 0);
+        for (uint32_t c = wa; c < we; ++c, blk += 32) {
+            uint4 v = nxt;
+            if (c + 1 < we && blk + 32 < p.nblocks) nxt = p.src[blk + 32];
+            if (DIR == 0) encrypt_block<NR>(v.x, v.y, v.z, v.w, T, K);
+            else decrypt_block<NR>(v.x, v.y, v.z, v.w, T, IS, K);
+            if (blk < p.nblocks) p.dst[blk] = v;
+        }
+        return;
     }
 
-    // the next chunk is fetched while this one is enciphered
-    uint4 nxt = blk < p.nblocks ? p.src[blk] : make_uint4(0, 0, 0, 0);
-    for (uint64_t c = c0; c < c1; ++c) {
-        const bool valid = blk < p.nblocks;
-        uint4 v = nxt;
-        if (c + 1 < c1 && blk + 32 < p.nblocks) nxt = p.src[blk + 32];
-        if (TWEAK) xor4(v, t0, t1, t2, t3);
-        if (DIR == 0) encrypt_block<NR>(v.x, v.y, v.z, v.w, T, K);
-        else decrypt_block<NR>(v.x, v.y, v.z, v.w, T, IS, K);
-        if (TWEAK) xor4(v, t0, t1, t2, t3);
-        if (valid) p.dst[blk] = v;
-        blk += 32;
-
-        if (TWEAK && c + 1 < c1) {
-            j += 32;
-            bool crossed = false;
-            if (j >= bps) {
-                uint32_t ns = j / bps;
-                srel += ns;
-                j -= ns * bps;
-                crossed = true;
-            }
-            if (__any_sync(0xffffffffu, srel >= 32)) {
-                uint32_t adv = __shfl_sync(0xffffffffu, srel, 0);
-                base += adv;
-                srel -= adv;
-                tweak_batch();
-            }
-            if (__any_sync(0xffffffffu, crossed)) {
-                uint32_t u0 = __shfl_sync(0xffffffffu, z0, srel & 31);
-                uint32_t u1 = __shfl_sync(0xffffffffu, z1, srel & 31);
-                uint32_t u2 = __shfl_sync(0xffffffffu, z2, srel & 31);
-                uint32_t u3 = __shfl_sync(0xffffffffu, z3, srel & 31);
-                if (crossed) {
-                    t0 = u0;
-                    t1 = u1;
-                    t2 = u2;
-                    t3 = u3;
-                    gf128_mul_xk(t0, t1, t2, t3, j);
+    const uint32_t bps = p.bps;
+    const bool shared = bps >= 32;  // the CTA forms the tweaks together
+    const uint32_t gthreads = shared ? (uint32_t)kBulkThreads : 32u;
+    const uint32_t gwarp = shared ? warp : 0u, gwarps = shared ? kWarps : 1u;
+    uint4* tw = reinterpret_cast<uint4*>(smem + (DIR == 0 ? kSmemEnc : kSmemDec)) + (shared ? 0u : warp * 32u);
+    auto group_sync = [&]() {
+        if (shared) __syncthreads();
+        else __syncwarp();
+    };
+    uint64_t c = first + (shared ? 0u : wa);
+    uint32_t left = shared ? own : we - wa;
+    bool again = false;
+    while (left) {
+        // the phase: as many chunks as have their units among gthreads
+        const uint64_t b0 = c << 5;
+        const uint64_t unit0 = div_small(b0, bps);
+        const uint32_t o = (uint32_t)(b0 - unit0 * bps);  // b0's place in unit0
+        const uint64_t fit = ((uint64_t)gthreads * bps - o) >> 5;  // >= 1
+        const uint32_t n = (uint32_t)min((uint64_t)min(left, 1u << 24), fit);
+        const uint32_t a = n * gwarp / gwarps, e = n * (gwarp + 1) / gwarps;
+        uint64_t blk = b0 + ((uint64_t)a << 5) + lane;
+        uint4 nxt = a < e && blk < p.nblocks ? p.src[blk] : make_uint4(0, 0, 0, 0);
+        if (again) group_sync();  // the last phase's tweaks have been read
+        again = true;
+        if ((uint64_t)gwarp * 32 * bps < (uint64_t)o + ((uint64_t)n << 5)) {  // units of this phase among this warp's
+            const uint64_t unit = p.first_sector + unit0 + gwarp * 32 + lane;
+            uint4 z = make_uint4((uint32_t)unit, (uint32_t)(unit >> 32), 0, 0);
+            if (DIR == 0) encrypt_block<NR>(z.x, z.y, z.z, z.w, T, TK);
+            else encrypt_block<NR>(z.x, z.y, z.z, z.w, TE, TK);
+            tw[gwarp * 32 + lane] = z;
+        }
+        group_sync();
+        if (a < e) {
+            const uint64_t q = (uint64_t)o + ((uint64_t)a << 5) + lane;
+            uint32_t u = (uint32_t)div_small(q, bps);  // unit of the phase
+            uint32_t j = (uint32_t)(q - (uint64_t)u * bps);
+            uint4 t = tw[u];
+            gf128_mul_xpow(t.x, t.y, t.z, t.w, j);
+            for (uint32_t i = a; i < e; ++i) {
+                uint4 v = nxt;
+                if (i + 1 < e && blk + 32 < p.nblocks) nxt = p.src[blk + 32];
+                xor4(v, t.x, t.y, t.z, t.w);
+                if (DIR == 0) encrypt_block<NR>(v.x, v.y, v.z, v.w, T, K);
+                else decrypt_block<NR>(v.x, v.y, v.z, v.w, T, IS, K);
+                xor4(v, t.x, t.y, t.z, t.w);
+                if (blk < p.nblocks) p.dst[blk] = v;
+                blk += 32;
+                if (i + 1 < e) {
+                    j += 32;
+                    if (j >= bps) {
+                        const uint32_t ns = shared ? 1u : j / bps;
+                        u += ns;
+                        j -= ns * bps;
+                        t = tw[u];
+                        gf128_mul_xk(t.x, t.y, t.z, t.w, j);
+                    } else {
+                        gf128_mul_x32(t.x, t.y, t.z, t.w);
+                    }
                 }
             }
-            if (!crossed) gf128_mul_x32(t0, t1, t2, t3);
         }
+        c += n;
+        left -= n;
     }
 }
 
@@ -608,6 +628,14 @@ __global__ void __launch_bounds__(kBulkThreads, 1) xts_cts_kernel(const __grid_c
 template <class P>
 using KernelFn = void (*)(P);
 
+// CTAs for a run of 32-block chunks: one per SM, and four chunks each (one per
+// SM quarter) before fewer are used.  Filling a CTA's warps first instead left
+// most SMs idle in small calls: 1 MiB ran on 64 of them.
+inline int grid_for_chunks(uint64_t chunks, int num_sms) {
+    const uint64_t ctas = (chunks + 3) / 4;
+    return (int)(ctas < (uint64_t)num_sms ? (ctas ? ctas : 1) : num_sms);
+}
+
 inline int grid_for(uint64_t warp_items, int num_sms) {
     // warp_items: how many warp-sized work items exist; at least one per warp.
     uint64_t ctas = (warp_items + (kBulkThreads / 32) - 1) / (kBulkThreads / 32);
@@ -629,6 +657,10 @@ KernelFn<BulkParams> bulk_fn(int nr, int dir, bool tweak) {
         case 14: return pick_bulk<14>(dir, tweak);
         default: return nullptr;
     }
+}
+
+size_t bulk_smem(int dir, bool tweak) {
+    return (dir == 0 ? kSmemEnc : kSmemDec) + (tweak ? kBulkThreads * 16 : 0);
 }
 
 KernelFn<CtsParams> cts_fn(int nr, int dir) {
@@ -712,7 +744,7 @@ cudaError_t configure_kernels() {
         for (int dir = 0; dir < 2; dir++) {
             for (bool tw : {false, true}) {
                 cudaError_t e = cudaFuncSetAttribute(bulk_fn(nr, dir, tw), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)(dir == 0 ? kSmemEnc : kSmemDec));
+                                                     (int)bulk_smem(dir, tw));
                 if (e != cudaSuccess) return e;
             }
         }
@@ -742,11 +774,16 @@ cudaError_t upload_tables(const uint32_t* te0, const uint32_t* td0, const uint32
     return e;
 }
 
-static cudaError_t launch_bulk(const BulkParams& p, int nr, int dir, bool tweak, int num_sms, cudaStream_t s) {
+static cudaError_t launch_bulk(const BulkParams& params, int nr, int dir, bool tweak, int num_sms, cudaStream_t s) {
     auto fn = bulk_fn(nr, dir, tweak);
     if (!fn) return cudaErrorInvalidValue;
-    int grid = grid_for((p.nblocks + 31) / 32, num_sms);
-    fn<<<grid, kBulkThreads, dir == 0 ? kSmemEnc : kSmemDec, s>>>(p);
+    BulkParams p = params;
+    const uint64_t chunks = (p.nblocks + 31) / 32;
+    const int grid = grid_for_chunks(chunks, num_sms);
+    if (chunks / grid >= 0xffffffffull) return cudaErrorInvalidValue;
+    p.cta_chunks = (uint32_t)(chunks / grid);
+    p.cta_rest = (uint32_t)(chunks % grid);
+    fn<<<grid, kBulkThreads, bulk_smem(dir, tweak), s>>>(p);
     return cudaGetLastError();
 }
 

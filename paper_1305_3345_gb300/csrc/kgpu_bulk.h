@@ -53,6 +53,8 @@ struct BulkParams {
     uint4* dst;
     uint64_t nblocks;       // 16-byte blocks in the buffer
     uint32_t bps;           // blocks per data unit (XTS)
+    uint32_t cta_rest;      // set by the launch: CTA b has cta_chunks 32-block chunks,
+    uint32_t cta_chunks;    // one more if b < cta_rest
     uint32_t pad0;
     uint64_t first_sector;  // number of the first data unit (XTS)
     uint32_t rk[kMaxRoundKeyWords];  // data key schedule (encryption or decryption order)

@@ -1,0 +1,47 @@
+"""How the bulk kernels split a buffer over CTAs and warps, at the sizes where
+the split changes, bit-exact against the CPU oracle: XTS with tweaks formed by
+the whole CTA (units of at least 512 B) or by each warp (smaller units), one
+phase or several, and chunk counts around one CTA's and one SM's share."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as w
+from conftest import to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+def sms():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def run_xts(ctx, key, dir, data, du, first, in_place):
+    kh = ctx.setkey(key, True)
+    try:
+        src = to_dev(data)
+        dst = src if in_place else src.new_empty(src.shape)
+        ctx.xts_crypt(kh, dir, src, dst, du, first)
+        return to_np(dst)
+    finally:
+        ctx.delkey(kh)
+
+
+@pytest.mark.parametrize("dir", [0, 1])
+@pytest.mark.parametrize("du,units", [
+    (512, lambda s: s * 1024 + 3 * s + 1),   # a phase holds 1,024 of them: two phases a CTA, uneven shares
+    (528, lambda s: s * 1024 + 2 * s + 5),   # 33 blocks: units straddle chunks and phases
+    (4096, lambda s: 1),                     # one CTA, eight chunks
+    (4096, lambda s: s // 2 + 1),            # four chunks a CTA: the last grid below one CTA per SM
+    (496, lambda s: 9 * s + 1),              # 31 blocks: formed by each warp, several phases a warp
+    (16, lambda s: 40 * s + 7),              # every block a unit: one chunk a phase
+])
+def test_xts_phases(ctx, dir, du, units):
+    n = units(sms())
+    key = w.xts_key(31, 256 if du != 512 else 128)
+    first = 2**40 + 11
+    data = w.seeded_bytes(31 + du, w.STREAM_DATA, du * n)
+    ref = oracle.xts(key, dir, data, du, first)
+    for in_place in (False, True):
+        assert np.array_equal(run_xts(ctx, key, dir, data, du, first, in_place), ref), (du, n, in_place)
