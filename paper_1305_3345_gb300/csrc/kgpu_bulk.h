@@ -68,6 +68,8 @@ struct CbcParams {
     const uint4* ivs;       // one per page
     uint64_t npages;
     uint32_t bpp;           // blocks per page
+    uint32_t cta_rest;      // set by the decryption launch: CTA b has cta_items pages or
+    uint32_t cta_items;     // chunks, one more if b < cta_rest
     uint32_t pad0;
     uint32_t rk[kMaxRoundKeyWords];
 };

@@ -1,5 +1,6 @@
 """How the bulk kernels split a buffer over CTAs and warps, at the sizes where
-the split changes, bit-exact against the CPU oracle: XTS with tweaks formed by
+the split changes, bit-exact against the CPU oracle: CBC decryption out of place
+(chunks) and in place (pages), and XTS with tweaks formed by
 the whole CTA (units of at least 512 B) or by each warp (smaller units), one
 phase or several, and chunk counts around one CTA's and one SM's share."""
 import numpy as np
@@ -45,3 +46,30 @@ def test_xts_phases(ctx, dir, du, units):
     ref = oracle.xts(key, dir, data, du, first)
     for in_place in (False, True):
         assert np.array_equal(run_xts(ctx, key, dir, data, du, first, in_place), ref), (du, n, in_place)
+
+
+@pytest.mark.parametrize("page,npages", [
+    (4096, lambda s: 1),
+    (4096, lambda s: s + 1),                 # in place: two pages on one CTA
+    (4096, lambda s: 4 * s + 3),             # about one chunk a warp
+    (512, lambda s: 32 * s + 7),             # a page is a chunk
+    (496, lambda s: 33 * s + 2),             # pages straddle chunks, warps and CTAs
+    (16, lambda s: 128 * s + 5),             # every block starts a page
+    (8 * 4096 + 48, lambda s: 3),            # long pages over many warps
+])
+def test_cbc_decrypt_split(ctx, page, npages):
+    n = npages(sms())
+    key = w.single_key(32, 192)
+    data = w.seeded_bytes(32 + page, w.STREAM_DATA, page * n)
+    ivs = w.page_ivs(32 + page, n)
+    ref = oracle.cbc(key, 1, data, page, ivs)
+    kh = ctx.setkey(key, False)
+    try:
+        iv = to_dev(np.ascontiguousarray(ivs).reshape(-1))
+        for in_place in (False, True):
+            src = to_dev(data)
+            dst = src if in_place else src.new_empty(src.shape)
+            ctx.cbc_decrypt(kh, src, dst, page, iv)
+            assert np.array_equal(to_np(dst), ref), (page, n, in_place)
+    finally:
+        ctx.delkey(kh)
