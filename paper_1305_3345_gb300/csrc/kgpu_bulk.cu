@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <mutex>
 
 #include "aes_device.cuh"
@@ -326,6 +327,94 @@ __global__ void __launch_bounds__(kBulkThreads, 1) cbc_enc_kernel(const __grid_c
     }
 }
 
+
+// ---------------------------------------------------------------------------
+// CBC encryption with a page's chain split over LANES = 4 or 2 lanes, for
+// calls whose time is a chain's latency.  A lane holds one or two columns of
+// its page's state; each round it takes the others from its neighbours by
+// shuffle and makes 4 or 8 lookups of its own, with its columns of the round
+// keys in registers.  A lane that holds a whole page makes 16 lookups in a row
+// before the next round can start: 107 cycles a round, against 77 with four
+// lanes and 78 with two.  Per round, four lanes spend 7 operations of the
+// shared-memory path on 8 pages and two spend 10 on 16, where one lane per
+// page spends 16 on 32: each form loses once that path is the bound (see
+// launch_cbc_enc).
+// ---------------------------------------------------------------------------
+template <int NR, int LANES>
+__global__ void __launch_bounds__(kCbcSplitThreads, 1) cbc_enc_split_kernel(const __grid_constant__ CbcParams p) {
+    extern __shared__ __align__(128) char smem[];
+    if (!smem_layout_ok(smem)) return;
+    fill_enc(smem);
+    constexpr int kCols = 4 / LANES;              // columns per lane
+    constexpr uint32_t kPages = 32 / LANES;       // pages per warp
+    using Piece = std::conditional_t<kCols == 1, uint32_t, uint2>;
+    const uint32_t lane = lane_id();
+    const uint32_t c = lane & (LANES - 1u), team = lane & ~(LANES - 1u);
+    const Rep4 T{lane * 4u, lane * 4u + 128u};
+    uint32_t k[NR + 1][kCols];
+#pragma unroll
+    for (int r = 0; r <= NR; r++)
+#pragma unroll
+        for (int i = 0; i < kCols; i++) k[r][i] = p.rk[4 * r + kCols * c + i];
+    const uint32_t bpp = p.bpp;
+    const uint64_t ngroups = (p.npages + kPages - 1) / kPages;
+    __syncthreads();
+
+    for (uint64_t g = interleaved_warp(); g < ngroups; g += total_warps()) {
+        // lanes without a page step along, loads and stores predicated off
+        const uint64_t page = g * kPages + lane / LANES;
+        const bool valid = page < p.npages;
+        const uint64_t at = (valid ? page : 0) * bpp * LANES + c;  // in pieces
+        const Piece* in = reinterpret_cast<const Piece*>(p.src) + at;
+        Piece* out = reinterpret_cast<Piece*>(p.dst) + at;
+        uint32_t s[4];  // this lane's columns, then the next lanes'
+        auto fetch = [&](const Piece* from, bool ok, uint32_t (&v)[kCols]) {
+            Piece w{};
+            if (ok) w = *from;
+            if constexpr (kCols == 1) {
+                v[0] = w;
+            } else {
+                v[0] = w.x;
+                v[1] = w.y;
+            }
+        };
+        uint32_t x[kCols], q[4][kCols];
+        fetch(reinterpret_cast<const Piece*>(p.ivs) + (valid ? page : 0) * LANES + c, valid, x);
+        // the chain is sequential, so plaintext is fetched four blocks ahead
+#pragma unroll
+        for (uint32_t i = 0; i < 4; i++) fetch(in + (size_t)LANES * i, valid && i < bpp, q[i]);
+        for (uint32_t i = 0; i < bpp; ++i) {
+#pragma unroll
+            for (int h = 0; h < kCols; h++) {
+                s[h] = x[h] ^ q[0][h] ^ k[0][h];
+                q[0][h] = q[1][h];
+                q[1][h] = q[2][h];
+                q[2][h] = q[3][h];
+            }
+            fetch(in + (size_t)LANES * (i + 4), valid && i + 4 < bpp, q[3]);
+#pragma unroll
+            for (int r = 1; r <= NR; r++) {
+#pragma unroll
+                for (int h = kCols; h < 4; h++)
+                    s[h] = __shfl_sync(0xffffffffu, s[h % kCols], team | ((c + h / kCols) & (LANES - 1u)));
+#pragma unroll
+                for (int h = 0; h < kCols; h++) {
+                    const uint32_t s0 = s[h], s1 = s[h + 1], s2 = s[(h + 2) & 3], s3 = s[(h + 3) & 3];
+                    if (r < NR)
+                        x[h] = T.t<0, 0>(s0) ^ k[r][h] ^ T.t<1, 1>(s1) ^ T.t<2, 2>(s2) ^ T.t<3, 3>(s3);
+                    else  // S(x) from the byte of table (r+3)%4 that holds it unscaled
+                        x[h] = merge_bytes(T.t<3, 0>(s0), T.t<0, 1>(s1), T.t<1, 2>(s2), T.t<2, 3>(s3)) ^ k[r][h];
+                }
+#pragma unroll
+                for (int h = 0; h < kCols; h++) s[h] = x[h];
+            }
+            if (valid) {
+                if constexpr (kCols == 1) out[(size_t)LANES * i] = x[0];
+                else out[(size_t)LANES * i] = make_uint2(x[0], x[1]);
+            }
+        }
+    }
+}
 
 // ---------------------------------------------------------------------------
 // CBC encryption, staged.  The chains are the same (one page per lane), but a
@@ -672,6 +761,15 @@ KernelFn<CtsParams> cts_fn(int nr, int dir) {
     }
 }
 
+KernelFn<CbcParams> cbc_enc_split_fn(int nr, int lanes) {
+    switch (nr) {
+        case 10: return lanes == 4 ? cbc_enc_split_kernel<10, 4> : cbc_enc_split_kernel<10, 2>;
+        case 12: return lanes == 4 ? cbc_enc_split_kernel<12, 4> : cbc_enc_split_kernel<12, 2>;
+        case 14: return lanes == 4 ? cbc_enc_split_kernel<14, 4> : cbc_enc_split_kernel<14, 2>;
+        default: return nullptr;
+    }
+}
+
 KernelFn<CbcParams> cbc_enc_staged_fn(int nr) {
     switch (nr) {
         case 10: return cbc_enc_staged_kernel<10>;
@@ -753,6 +851,11 @@ cudaError_t configure_kernels() {
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(cbc_fn(nr, false), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDec);
         if (e != cudaSuccess) return e;
+        for (int lanes : {2, 4}) {
+            e = cudaFuncSetAttribute(cbc_enc_split_fn(nr, lanes), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kSmemEnc);
+            if (e != cudaSuccess) return e;
+        }
         e = cudaFuncSetAttribute(cbc_enc_staged_fn(nr), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kSmemEncStaged);
         if (e != cudaSuccess) return e;
@@ -880,6 +983,22 @@ bool page_tile_maps(CbcTmaParams* t, const CbcParams& p) {
 }
 
 cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t s) {
+    // Few pages are a chain's latency, which two or four lanes per page
+    // shorten; many are the lookups' rate, which one lane per page uses best.
+    // 4-KiB pages, AES-128, one / two / four lanes: 8 pages per SM 145 / 107 /
+    // 103 us, 32 pages 145 / 109 / 107, 64 pages 147 / 121 / 121, 128 pages 153
+    // / 152 / 180, 160 pages 206 / 182 / 288, 192 pages 208 / 207 / 295, 224
+    // pages 215 / 248 / 316.  Pages that cannot be staged cross later (4112 B,
+    // AES-256: 224 pages 299 / 286, 256 pages 306 / 309).
+    const uint64_t sms = (uint64_t)(num_sms > 0 ? num_sms : 1);
+    const int lanes = p.npages <= 32 * sms ? 4 : p.npages <= (p.bpp % kStageBlocks ? 240 : 192) * sms ? 2 : 1;
+    if (lanes > 1) {
+        auto fn = cbc_enc_split_fn(nr, lanes);
+        if (!fn) return cudaErrorInvalidValue;
+        const uint64_t teams = (p.npages + 32 / lanes - 1) / (32 / lanes);
+        fn<<<(int)std::min<uint64_t>(teams, sms), kCbcSplitThreads, kSmemEnc, s>>>(p);
+        return cudaGetLastError();
+    }
     // The tensor tiles take a seventh of the staging traffic off the
     // shared-memory path, which pays once that path is the bound: from 12
     // groups of 32 pages per SM (measured at 4-KiB pages: 8 groups per SM
@@ -887,7 +1006,7 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
     // 389 against 355 us).  Below that a launch is a chain's latency either
     // way, and the tiles' two tensor maps would only add host time.
     const uint64_t groups = (p.npages + 31) / 32;
-    if (p.bpp % kStageBlocks == 0 && groups >= 12ull * (uint64_t)(num_sms > 0 ? num_sms : 1)) {
+    if (p.bpp % kStageBlocks == 0 && groups >= 12 * sms) {
         CbcTmaParams t;
         std::memset(&t, 0, sizeof(t));
         auto fn = cbc_enc_tma_fn(nr);

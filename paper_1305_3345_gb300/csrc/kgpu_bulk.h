@@ -21,6 +21,9 @@ constexpr size_t kSmemDec = 3 * kRegionBytes;  // regions A, B, C
 // Threads per CTA of the bulk kernels (one CTA per SM).
 constexpr int kBulkThreads = 1024;
 
+// CBC encryption with a chain split over 2 or 4 lanes: at most 16 warps per CTA.
+constexpr int kCbcSplitThreads = 512;
+
 // Staged CBC encryption: up to 20 warps per CTA (96 registers a thread), each
 // with a 32-page x 8-block staging area (4608 B) after the two table regions.
 // The launch picks the warp count for the page count (cbc_enc_staged_warps).

@@ -1,6 +1,6 @@
 """How the bulk kernels split a buffer over CTAs and warps, at the sizes where
 the split changes, bit-exact against the CPU oracle: CBC decryption out of place
-(chunks) and in place (pages), and XTS with tweaks formed by
+(chunks) and in place (pages), CBC encryption with one, two or four lanes per page, and XTS with tweaks formed by
 the whole CTA (units of at least 512 B) or by each warp (smaller units), one
 phase or several, and chunk counts around one CTA's and one SM's share."""
 import numpy as np
@@ -71,5 +71,33 @@ def test_cbc_decrypt_split(ctx, page, npages):
             dst = src if in_place else src.new_empty(src.shape)
             ctx.cbc_decrypt(kh, src, dst, page, iv)
             assert np.array_equal(to_np(dst), ref), (page, n, in_place)
+    finally:
+        ctx.delkey(kh)
+
+
+@pytest.mark.parametrize("page,npages", [
+    (4096, lambda s: 1),
+    (48, lambda s: 32 * s),                  # four lanes a page: the largest call
+    (16, lambda s: 32 * s + 1),              # two lanes a page: the smallest, ragged team
+    (128, lambda s: 192 * s),                # two lanes: the largest of pages that can be staged
+    (128, lambda s: 192 * s + 1),            # one lane
+    (48, lambda s: 240 * s + 9),             # one lane, pages that cannot be staged
+    (80, lambda s: 240 * s - 3),             # two lanes: several waves of warps
+])
+@pytest.mark.parametrize("bits", [128, 192, 256])
+def test_cbc_encrypt_lanes(ctx, bits, page, npages):
+    n = npages(sms())
+    key = w.single_key(33, bits)
+    data = w.seeded_bytes(33 + page, w.STREAM_DATA, page * n)
+    ivs = w.page_ivs(33 + page, n)
+    ref = oracle.cbc(key, 0, data, page, ivs)
+    kh = ctx.setkey(key, False)
+    try:
+        iv = to_dev(np.ascontiguousarray(ivs).reshape(-1))
+        for in_place in (False, True):
+            src = to_dev(data)
+            dst = src if in_place else src.new_empty(src.shape)
+            ctx.cbc_encrypt_pages(kh, src, dst, page, iv)
+            assert np.array_equal(to_np(dst), ref), (bits, page, n, in_place)
     finally:
         ctx.delkey(kh)
