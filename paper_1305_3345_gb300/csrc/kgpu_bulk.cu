@@ -607,51 +607,134 @@ __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_tma_kernel(co
 // ---------------------------------------------------------------------------
 // XTS with ciphertext stealing (IEEE 1619-2007 5.3.2 encryption, 5.4.2
 // decryption) for data units of du bytes, du >= 16 and not a multiple of 16:
-// m full blocks and a final partial block of b bytes.  One warp per data unit:
-// full blocks 0..m-2 go to the lanes (block j with T * alpha^j), then lane 0
-// runs the stealing pair, the last full block and the partial block, which
-// depend on each other:
+// m full blocks and a final partial block of b bytes.  The last full block and
+// the partial block depend on each other:
 //   encryption: CC = enc(P_{m-1}, T a^{m-1});  C_m = CC[0..b);
 //               C_{m-1} = enc(P_m || CC[b..16), T a^m)
 //   decryption: PP = dec(C_{m-1}, T a^m);  P_m = PP[0..b);
 //               P_{m-1} = dec(C_m || PP[b..16), T a^{m-1})
-// Unit starts are only as aligned as u * du, so the unit's blocks move through
-// 16-, 4- or 1-byte accesses as its start allows.
+// A CTA owns a run of units and takes them in phases of one unit per thread:
+// the threads encipher the units' tweaks, then the m full blocks of all units
+// as one sequence of 32-block chunks split over the warps (the CC or PP of
+// each unit stays in shared memory), then the second block of the pair, one
+// unit per thread.  So every lane has a block in each of the three passes and
+// the lookups are the bound; with one warp per unit, two of the warp's 34
+// enciphering steps on a 520-byte unit worked for one lane only, one more for
+// the tweak, and a 100-byte unit filled 6 of 32 lanes.
+// 32,768 units of 520 B, AES-256: 120.4 -> 34.9 us (488.9 GB/s); 8,192 of 527 B,
+// decryption: 41.1 -> 18.5 us; 10,485 of 100 B, AES-128: 32.8 -> 8.2 us.
+//
+// Unit starts are only as aligned as u * du.  Units of a multiple of 8 bytes
+// move in 8-byte accesses; others are read as the two aligned 16-byte words
+// that hold a block and shifted into place, and written in the widest pieces
+// that their address allows.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 load_block(const uint8_t* q, uint32_t align) {
-    if (align == 16) return *reinterpret_cast<const uint4*>(q);
-    uint32_t w[4];
+__device__ __forceinline__ uint4 load_tail_word(const uint8_t* q, const uint8_t* end) {
+    // the aligned word at q, of which only the bytes before end are there
+    uint32_t w[4] = {0, 0, 0, 0};
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        if (align == 4) {
-            w[i] = reinterpret_cast<const uint32_t*>(q)[i];
-        } else {
-            w[i] = (uint32_t)q[4 * i] | (uint32_t)q[4 * i + 1] << 8 | (uint32_t)q[4 * i + 2] << 16 |
-                   (uint32_t)q[4 * i + 3] << 24;
-        }
-    }
+    for (int k = 0; k < 16; k++)
+        if (q + k < end) w[k >> 2] |= (uint32_t)q[k] << (8 * (k & 3));
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__device__ __forceinline__ void store_block(uint8_t* q, const uint4& v, uint32_t align) {
-    if (align == 16) {
-        *reinterpret_cast<uint4*>(q) = v;
+// The 16 bytes at q as loaded (lo, hi), and put in place by settle().
+struct RawBlock {
+    uint4 lo, hi;
+};
+
+__device__ __forceinline__ RawBlock load_raw(const uint8_t* q, const uint8_t* end, bool by8) {
+    RawBlock r;
+    r.hi = make_uint4(0, 0, 0, 0);
+    if (by8) {
+        const uint2 x = *reinterpret_cast<const uint2*>(q);
+        const uint2 y = q + 16 <= end ? *reinterpret_cast<const uint2*>(q + 8) : make_uint2(0, 0);
+        r.lo = make_uint4(x.x, x.y, y.x, y.y);
+        return r;
+    }
+    const uint32_t off = (uint32_t)((uintptr_t)q & 15u);
+    const uint8_t* a = q - off;
+    r.lo = a + 16 <= end ? *reinterpret_cast<const uint4*>(a) : load_tail_word(a, end);
+    if (off && a + 16 < end) r.hi = a + 32 <= end ? *reinterpret_cast<const uint4*>(a + 16) : load_tail_word(a + 16, end);
+    return r;
+}
+
+__device__ __forceinline__ uint4 settle(const RawBlock& r, const uint8_t* q, bool by8) {
+    if (by8) return r.lo;
+    const uint32_t off = (uint32_t)((uintptr_t)q & 15u), sh = (off & 3u) * 8u;
+    const bool s1 = (off & 4u) != 0, s2 = (off & 8u) != 0;
+    uint32_t w[8] = {r.lo.x, r.lo.y, r.lo.z, r.lo.w, r.hi.x, r.hi.y, r.hi.z, r.hi.w};
+#pragma unroll
+    for (int i = 0; i < 6; i++) w[i] = s2 ? w[i + 2] : w[i];
+#pragma unroll
+    for (int i = 0; i < 5; i++) w[i] = s1 ? w[i + 1] : w[i];
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                      __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+}
+
+__device__ __forceinline__ void store_any(uint8_t* q, const uint4& v, bool by8) {
+    if (by8) {
+        reinterpret_cast<uint2*>(q)[0] = make_uint2(v.x, v.y);
+        reinterpret_cast<uint2*>(q)[1] = make_uint2(v.z, v.w);
         return;
     }
+    const uint32_t k = (uint32_t)((uintptr_t)q & 3u);
+    if (k == 0) {
+        uint32_t* o = reinterpret_cast<uint32_t*>(q);
+        o[0] = v.x;
+        o[1] = v.y;
+        o[2] = v.z;
+        o[3] = v.w;
+        return;
+    }
+    const uint32_t h = 4 - k;  // bytes up to the first aligned word
+    if (h & 1u) {
+        q[0] = (uint8_t)v.x;
+        if (h == 3) *reinterpret_cast<uint16_t*>(q + 1) = (uint16_t)(v.x >> 8);
+    } else {
+        *reinterpret_cast<uint16_t*>(q) = (uint16_t)v.x;
+    }
+    uint32_t* o = reinterpret_cast<uint32_t*>(q + h);
+    o[0] = __funnelshift_r(v.x, v.y, 8 * h);
+    o[1] = __funnelshift_r(v.y, v.z, 8 * h);
+    o[2] = __funnelshift_r(v.z, v.w, 8 * h);
+    const uint32_t rest = v.w >> (8 * h);  // the last k bytes
+    uint8_t* t = q + 16 - k;
+    if (k & 2u) {
+        *reinterpret_cast<uint16_t*>(t) = (uint16_t)rest;
+        if (k == 3) t[2] = (uint8_t)(rest >> 16);
+    } else {
+        t[0] = (uint8_t)rest;
+    }
+}
+
+// The first b (< 16) bytes of v.
+__device__ __forceinline__ void store_part(uint8_t* q, const uint4& v, uint32_t b) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const bool by4 = ((uintptr_t)q & 3u) == 0;
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        if (align == 4) {
+    for (uint32_t i = 0; i < 4; i++) {
+        if (by4 && b >= 4 * i + 4) {
             reinterpret_cast<uint32_t*>(q)[i] = w[i];
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; k++) q[4 * i + k] = (uint8_t)(w[i] >> (8 * k));
+            for (uint32_t k = 0; k < 4; k++)
+                if (4 * i + k < b) q[4 * i + k] = (uint8_t)(w[i] >> (8 * k));
         }
     }
 }
 
+// Bytes [0, b) of x and [b, 16) of y.
+__device__ __forceinline__ uint4 splice(const uint4& x, const uint4& y, uint32_t b) {
+    auto word = [&](uint32_t xw, uint32_t yw, uint32_t i) {
+        const uint32_t mask = b >= 4 * i + 4 ? ~0u : b <= 4 * i ? 0u : (1u << (8 * (b - 4 * i))) - 1u;
+        return (xw & mask) | (yw & ~mask);
+    };
+    return make_uint4(word(x.x, y.x, 0), word(x.y, y.y, 1), word(x.z, y.z, 2), word(x.w, y.w, 3));
+}
+
 template <int NR, int DIR>
-__global__ void __launch_bounds__(kBulkThreads, 1) xts_cts_kernel(const __grid_constant__ CtsParams p) {
+__global__ void __launch_bounds__(kCtsThreads, 1) xts_cts_kernel(const __grid_constant__ CtsParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
     if (DIR == 0) fill_enc(smem);
@@ -659,66 +742,115 @@ __global__ void __launch_bounds__(kBulkThreads, 1) xts_cts_kernel(const __grid_c
     __syncthreads();
 
     const uint32_t lane = lane_id();
+    const uint32_t warp = threadIdx.x >> 5;
+    constexpr uint32_t kWarps = kCtsThreads / 32;
     const Rep4 T{lane * 4u, lane * 4u + 128u};
     const Rep1<2> IS{lane * 4u};
     const Rep1<2> TE{lane * 4u + 128u};
     const ParamKey K{p.rk};
     const ParamKey TK{p.tk};
-    const uint64_t m = p.du / 16;
-    const uint32_t b = (uint32_t)(p.du % 16);
+    uint4* tw = reinterpret_cast<uint4*>(smem + (DIR == 0 ? kSmemEnc : kSmemDec));  // E_K2 of the phase's units
+    uint4* cc = tw + kCtsThreads;                                                   // CC / PP of its units
 
-    auto block = [&](uint4& v, uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3) {
-        xor4(v, t0, t1, t2, t3);
+    const uint64_t du = p.du;
+    const uint32_t m = (uint32_t)(du / 16), b = (uint32_t)(du % 16);
+    const bool by8 = b == 8;
+    const uint8_t* end = p.src + p.units * du;
+    const uint64_t first = (uint64_t)p.cta_units * blockIdx.x + min((uint64_t)blockIdx.x, (uint64_t)p.cta_rest);
+    const uint64_t own = p.cta_units + (blockIdx.x < p.cta_rest ? 1u : 0u);
+    const uint32_t most = max(1u, min((uint32_t)kCtsThreads, (1u << 30) / m));  // units per phase
+
+    auto cipher = [&](uint4& v, const uint4& t) {
+        xor4(v, t.x, t.y, t.z, t.w);
         if (DIR == 0) encrypt_block<NR>(v.x, v.y, v.z, v.w, T, K);
         else decrypt_block<NR>(v.x, v.y, v.z, v.w, T, IS, K);
-        xor4(v, t0, t1, t2, t3);
+        xor4(v, t.x, t.y, t.z, t.w);
     };
 
-    for (uint64_t u = interleaved_warp(); u < p.units; u += total_warps()) {
-        const uint8_t* in = p.src + u * p.du;
-        uint8_t* out = p.dst + u * p.du;
-        const uint32_t off = (uint32_t)((uintptr_t)in & 15u);
-        const uint32_t align = off == 0 ? 16u : (off & 3u) == 0 ? 4u : 1u;
-        // E_K2(unit number) on every lane
-        const uint64_t unit = p.first_sector + u;
-        uint32_t z0 = (uint32_t)unit, z1 = (uint32_t)(unit >> 32), z2 = 0, z3 = 0;
-        if (DIR == 0) encrypt_block<NR>(z0, z1, z2, z3, T, TK);
-        else encrypt_block<NR>(z0, z1, z2, z3, TE, TK);
-        // blocks 0..m-2, lane-strided
-        uint32_t t0 = z0, t1 = z1, t2 = z2, t3 = z3;
-        gf128_mul_xk(t0, t1, t2, t3, lane);
-        for (uint64_t j = lane; j + 1 < m; j += 32) {
-            uint4 v = load_block(in + 16 * j, align);
-            block(v, t0, t1, t2, t3);
-            store_block(out + 16 * j, v, align);
-            gf128_mul_x32(t0, t1, t2, t3);
+    for (uint64_t done = 0; done < own;) {
+        const uint32_t n = (uint32_t)min(own - done, (uint64_t)most);
+        const uint64_t unit0 = first + done;
+        if (done) __syncthreads();  // the last phase's tw and cc have been read
+        if (warp * 32 < n) {
+            const uint64_t unit = p.first_sector + unit0 + threadIdx.x;
+            uint4 z = make_uint4((uint32_t)unit, (uint32_t)(unit >> 32), 0, 0);
+            if (DIR == 0) encrypt_block<NR>(z.x, z.y, z.z, z.w, T, TK);
+            else encrypt_block<NR>(z.x, z.y, z.z, z.w, TE, TK);
+            tw[threadIdx.x] = z;
         }
-        // the stealing pair: tweaks T a^{m-1} (a*) and T a^m (c*)
-        if (lane == 0) {
-            uint32_t a0 = z0, a1 = z1, a2 = z2, a3 = z3;
-            gf128_mul_xpow(a0, a1, a2, a3, (uint32_t)(m - 1));
-            uint32_t c0 = a0, c1 = a1, c2 = a2, c3 = a3;
-            gf128_mul_xk(c0, c1, c2, c3, 1);
-            uint4 x = load_block(in + 16 * (m - 1), align);
-            const uint8_t* tail = in + 16 * m;
-            // both inputs are read before anything is written (in-place calls)
-            uint32_t yw[4] = {0, 0, 0, 0};
-            if (DIR == 0) block(x, a0, a1, a2, a3);  // CC
-            else block(x, c0, c1, c2, c3);           // PP
-            const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int k = 0; k < 16; k++) {
-                const uint32_t byte = (uint32_t)k < b ? (uint32_t)tail[k] : (xw[k >> 2] >> (8 * (k & 3))) & 0xffu;
-                yw[k >> 2] |= byte << (8 * (k & 3));
+        __syncthreads();
+
+        // the full blocks: block j of unit u is item u * m + j
+        const uint64_t items = (uint64_t)n * m;
+        const uint32_t chunks = (uint32_t)((items + 31) >> 5);
+        const uint32_t a = (uint32_t)((uint64_t)chunks * warp / kWarps);
+        const uint32_t e = (uint32_t)((uint64_t)chunks * (warp + 1) / kWarps);
+        if (a < e) {
+            uint64_t q = ((uint64_t)a << 5) + lane;
+            const bool some = q < items;
+            uint32_t u = some ? (uint32_t)div_small(q, m) : 0u;
+            uint32_t j = some ? (uint32_t)(q - (uint64_t)u * m) : 0u;
+            uint64_t off = (unit0 + u) * du + 16ull * j;
+            uint4 t = tw[u];
+            gf128_mul_xpow(t.x, t.y, t.z, t.w, j);
+            RawBlock nxt{};
+            if (some) nxt = load_raw(p.src + off, end, by8);
+            for (uint32_t i = a; i < e; ++i) {
+                uint4 v = settle(nxt, p.src + off, by8);
+                const bool valid = q < items;
+                // where this lane goes next; its block is fetched meanwhile
+                uint32_t un = u, jn = j + 32;
+                uint64_t offn = off + 512;
+                q += 32;
+                const bool more = i + 1 < e && q < items;
+                const bool crossed = jn >= m;
+                if (more && crossed) {
+                    const uint32_t ns = m >= 32 ? 1u : jn / m;
+                    un += ns;
+                    jn -= ns * m;
+                    offn = (unit0 + un) * du + 16ull * jn;
+                }
+                if (more) nxt = load_raw(p.src + offn, end, by8);
+                const bool last = j + 1 == m;
+                uint4 tv = t;
+                if (DIR == 1 && last) gf128_mul_xk(tv.x, tv.y, tv.z, tv.w, 1);
+                cipher(v, tv);
+                if (valid) {
+                    if (last) cc[u] = v;
+                    else store_any(p.dst + off, v, by8);
+                }
+                if (more) {
+                    if (crossed) {
+                        t = tw[un];
+                        gf128_mul_xk(t.x, t.y, t.z, t.w, jn);
+                    } else {
+                        gf128_mul_x32(t.x, t.y, t.z, t.w);
+                    }
+                }
+                u = un;
+                j = jn;
+                off = offn;
             }
-            uint4 y = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-            if (DIR == 0) block(y, c0, c1, c2, c3);  // C_{m-1}
-            else block(y, a0, a1, a2, a3);           // P_{m-1}
-            store_block(out + 16 * (m - 1), y, align);
-#pragma unroll
-            for (int k = 0; k < 16; k++)
-                if ((uint32_t)k < b) out[16 * m + k] = (uint8_t)(xw[k >> 2] >> (8 * (k & 3)));
         }
+        __syncthreads();
+
+        // the pair's second block, one unit per thread
+        if (warp * 32 < n) {
+            const bool valid = threadIdx.x < n;
+            const uint32_t u = valid ? threadIdx.x : 0u;
+            const uint64_t off = (unit0 + u) * du + 16ull * (m - 1);
+            uint4 t = tw[u];
+            gf128_mul_xpow(t.x, t.y, t.z, t.w, DIR == 0 ? m : m - 1);
+            const uint4 x = cc[u];
+            const uint8_t* tail = p.src + off + 16;
+            uint4 y = splice(settle(load_raw(tail, end, by8), tail, by8), x, b);
+            cipher(y, t);
+            if (valid) {
+                store_part(p.dst + off + 16, x, b);
+                store_any(p.dst + off, y, by8);
+            }
+        }
+        done += n;
     }
 }
 
@@ -752,10 +884,11 @@ size_t bulk_smem(int dir, bool tweak) {
     return (dir == 0 ? kSmemEnc : kSmemDec) + (tweak ? kBulkThreads * 16 : 0);
 }
 
+size_t cts_smem(int dir) { return (dir == 0 ? kSmemEnc : kSmemDec) + kCtsThreads * 32; }
+
 KernelFn<CtsParams> cts_fn(int nr, int dir) {
     switch (nr) {
         case 10: return dir ? xts_cts_kernel<10, 1> : xts_cts_kernel<10, 0>;
-        case 12: return dir ? xts_cts_kernel<12, 1> : xts_cts_kernel<12, 0>;
         case 14: return dir ? xts_cts_kernel<14, 1> : xts_cts_kernel<14, 0>;
         default: return nullptr;
     }
@@ -862,8 +995,8 @@ cudaError_t configure_kernels() {
         e = cudaFuncSetAttribute(cbc_enc_tma_fn(nr), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemEncTma);
         if (e != cudaSuccess) return e;
         for (int dir = 0; dir < 2; dir++) {
-            e = cudaFuncSetAttribute(cts_fn(nr, dir), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(dir == 0 ? kSmemEnc : kSmemDec));
+            if (!cts_fn(nr, dir)) continue;  // there is no XTS-AES-192
+            e = cudaFuncSetAttribute(cts_fn(nr, dir), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cts_smem(dir));
             if (e != cudaSuccess) return e;
         }
     }
@@ -915,10 +1048,13 @@ cudaError_t launch_cbc_dec(const CbcParams& p, int nr, int num_sms, cudaStream_t
 cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cudaStream_t s) {
     auto fn = cts_fn(nr, dir);
     if (!fn) return cudaErrorInvalidValue;
-    const uint64_t warps = kBulkThreads / 32;
-    const uint64_t ctas = (p.units + warps - 1) / warps;
-    const int grid = (int)(ctas < (uint64_t)num_sms ? (ctas ? ctas : 1) : num_sms);
-    fn<<<grid, kBulkThreads, dir == 0 ? kSmemEnc : kSmemDec, s>>>(p);
+    CtsParams q = p;
+    // a CTA per SM from four 32-block chunks each, and never less than a unit
+    const uint64_t chunks = (p.units * (p.du / 16) + 31) / 32;
+    const int grid = (int)std::min<uint64_t>(p.units, grid_for_chunks(chunks, num_sms));
+    q.cta_units = p.units / grid;
+    q.cta_rest = (uint32_t)(p.units % grid);
+    fn<<<grid, kCtsThreads, cts_smem(dir), s>>>(q);
     return cudaGetLastError();
 }
 

@@ -24,6 +24,12 @@ constexpr int kBulkThreads = 1024;
 // CBC encryption with a chain split over 2 or 4 lanes: at most 16 warps per CTA.
 constexpr int kCbcSplitThreads = 512;
 
+// XTS with ciphertext stealing: 24 warps (80 registers a thread, for the two
+// words of an unaligned block in flight), two 16-byte words per thread after
+// the tables.
+constexpr int kCtsThreads = 768;
+static_assert(kSmemDec + kCtsThreads * 32 <= 232448, "ciphertext stealing exceeds the 227-KB shared-memory limit");
+
 // Staged CBC encryption: up to 20 warps per CTA (96 registers a thread), each
 // with a 32-page x 8-block staging area (4608 B) after the two table regions.
 // The launch picks the warp count for the page count (cbc_enc_staged_warps).
@@ -98,6 +104,9 @@ struct CtsParams {
     uint64_t units;
     uint64_t du;
     uint64_t first_sector;
+    uint64_t cta_units;  // set by the launch: CTA b has cta_units units, one more if b < cta_rest
+    uint32_t cta_rest;
+    uint32_t pad0;
     uint32_t rk[kMaxRoundKeyWords];
     uint32_t tk[kMaxRoundKeyWords];
 };

@@ -1,8 +1,10 @@
-"""How the bulk kernels split a buffer over CTAs and warps, at the sizes where
-the split changes, bit-exact against the CPU oracle: CBC decryption out of place
-(chunks) and in place (pages), CBC encryption with one, two or four lanes per page, and XTS with tweaks formed by
-the whole CTA (units of at least 512 B) or by each warp (smaller units), one
-phase or several, and chunk counts around one CTA's and one SM's share."""
+"""How the bulk kernels split a buffer over CTAs, warps and lanes, at the sizes
+where the split changes, bit-exact against the CPU oracle: XTS with tweaks
+formed by the whole CTA (units of at least 512 B) or by each warp (smaller
+units), one phase or several; XTS units that end in ciphertext stealing, in
+phases of one unit per thread and at every alignment; CBC decryption out of
+place (chunks) and in place (pages); CBC encryption with one, two or four lanes
+per page."""
 import numpy as np
 import pytest
 
@@ -101,3 +103,23 @@ def test_cbc_encrypt_lanes(ctx, bits, page, npages):
             assert np.array_equal(to_np(dst), ref), (bits, page, n, in_place)
     finally:
         ctx.delkey(kh)
+
+
+@pytest.mark.parametrize("dir", [0, 1])
+@pytest.mark.parametrize("du,units", [
+    (24, lambda s: 768 * s + 2 * s + 1),     # 8-byte accesses, two phases a CTA
+    (19, lambda s: 768 * s + 5),             # byte alignment, one block a unit
+    (18, lambda s: 5 * s),                   # 2-byte alignment
+    (20, lambda s: 1),                       # one unit, the whole buffer 20 bytes
+    (520, lambda s: 4 * s + 1),              # 32 blocks and a half: a chunk a unit
+    (1037, lambda s: 97),                    # 64 blocks and 13 bytes, fewer units than SMs
+    (70002, lambda s: 3),                    # long units
+])
+def test_xts_stealing_phases(ctx, dir, du, units):
+    n = units(sms())
+    key = w.xts_key(34, 128 if du % 2 else 256)
+    first = 2**33 + 5
+    data = w.seeded_bytes(34 + du, w.STREAM_DATA, du * n)
+    ref = oracle.xts(key, dir, data, du, first)
+    for in_place in (False, True):
+        assert np.array_equal(run_xts(ctx, key, dir, data, du, first, in_place), ref), (du, n, in_place)
