@@ -77,6 +77,19 @@ __device__ __forceinline__ void xor4(uint4& v, uint32_t a, uint32_t b, uint32_t 
     v.w ^= d;
 }
 
+// Programmatic dependent launch.  A launch's tables do not depend on the work
+// queued before it, so the kernels are launched with programmatic stream
+// serialisation: next_may_start() lets the next such launch of the stream put
+// its CTAs on SMs that have room and fill their tables while this one runs,
+// and wait_for_previous() holds every CTA, before it touches a caller's buffer,
+// until all earlier work of the stream has completed and its writes are
+// visible.  Every CTA waits, so a launch never completes before the one it
+// follows.  GPU time of back-to-back calls without and with it: 4 KiB of
+// AES-256-XTS 7.2 / 4.4 us, 1 MiB 8.2 / 5.5, 16 MiB 30.8 / 28.4, 64 MiB of
+// AES-128-CBC decryption 81.9 / 77.5.
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // a / b where a rarely needs more than 32 bits.
 __device__ __forceinline__ uint64_t div_small(uint64_t a, uint32_t b) {
     return (a >> 32) == 0 ? (uint64_t)((uint32_t)a / b) : a / b;
@@ -103,8 +116,10 @@ template <int NR, int DIR, bool TWEAK>
 __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_constant__ BulkParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;  // uniform over the CTA; refused at init
+    next_may_start();
     if (DIR == 0) fill_enc(smem);
     else fill_dec<TWEAK>(smem);
+    wait_for_previous();
     __syncthreads();
 
     const uint32_t lane = lane_id();
@@ -221,7 +236,9 @@ template <int NR>
 __global__ void __launch_bounds__(kBulkThreads, 1) cbc_dec_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
+    next_may_start();
     fill_dec<false>(smem);
+    wait_for_previous();
 
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
@@ -291,7 +308,9 @@ template <int NR>
 __global__ void __launch_bounds__(kBulkThreads, 1) cbc_enc_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
+    next_may_start();
     fill_enc(smem);
+    wait_for_previous();
     __syncthreads();
 
     const uint32_t lane = lane_id();
@@ -344,7 +363,9 @@ template <int NR, int LANES>
 __global__ void __launch_bounds__(kCbcSplitThreads, 1) cbc_enc_split_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
+    next_may_start();
     fill_enc(smem);
+    wait_for_previous();
     constexpr int kCols = 4 / LANES;              // columns per lane
     constexpr uint32_t kPages = 32 / LANES;       // pages per warp
     using Piece = std::conditional_t<kCols == 1, uint32_t, uint2>;
@@ -435,7 +456,9 @@ template <int NR>
 __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_staged_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
+    next_may_start();
     fill_enc(smem);
+    wait_for_previous();
     __syncthreads();
 
     const uint32_t lane = lane_id();
@@ -542,6 +565,7 @@ template <int NR>
 __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_tma_kernel(const __grid_constant__ CbcTmaParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
+    next_may_start();
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
     // kSmemBase + kSmemEnc + warp * 4096: 1024-byte aligned in the shared
@@ -555,6 +579,7 @@ __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_tma_kernel(co
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor copies see it initialised
     }
     fill_enc(smem);
+    wait_for_previous();
     __syncthreads();
 
     const Rep4 T{lane * 4u, lane * 4u + 128u};
@@ -737,8 +762,10 @@ template <int NR, int DIR>
 __global__ void __launch_bounds__(kCtsThreads, 1) xts_cts_kernel(const __grid_constant__ CtsParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
+    next_may_start();
     if (DIR == 0) fill_enc(smem);
     else fill_dec<true>(smem);
+    wait_for_previous();
     __syncthreads();
 
     const uint32_t lane = lane_id();
@@ -856,6 +883,22 @@ __global__ void __launch_bounds__(kCtsThreads, 1) xts_cts_kernel(const __grid_co
 
 template <class P>
 using KernelFn = void (*)(P);
+
+// Launch with programmatic stream serialisation (see next_may_start).
+template <class P>
+cudaError_t launch(KernelFn<P> fn, int grid, int threads, size_t smem, cudaStream_t s, const P& p) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, p);
+}
 
 // CTAs for a run of 32-block chunks: one per SM, and four chunks each (one per
 // SM quarter) before fewer are used.  Filling a CTA's warps first instead left
@@ -1019,8 +1062,7 @@ static cudaError_t launch_bulk(const BulkParams& params, int nr, int dir, bool t
     if (chunks / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     p.cta_chunks = (uint32_t)(chunks / grid);
     p.cta_rest = (uint32_t)(chunks % grid);
-    fn<<<grid, kBulkThreads, bulk_smem(dir, tweak), s>>>(p);
-    return cudaGetLastError();
+    return launch(fn, grid, kBulkThreads, bulk_smem(dir, tweak), s, p);
 }
 
 cudaError_t launch_xts(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s) {
@@ -1041,8 +1083,7 @@ cudaError_t launch_cbc_dec(const CbcParams& p, int nr, int num_sms, cudaStream_t
     if (items / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     q.cta_items = (uint32_t)(items / grid);
     q.cta_rest = (uint32_t)(items % grid);
-    fn<<<grid, kBulkThreads, kSmemDec, s>>>(q);
-    return cudaGetLastError();
+    return launch(fn, grid, kBulkThreads, kSmemDec, s, q);
 }
 
 cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cudaStream_t s) {
@@ -1054,8 +1095,7 @@ cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cud
     const int grid = (int)std::min<uint64_t>(p.units, grid_for_chunks(chunks, num_sms));
     q.cta_units = p.units / grid;
     q.cta_rest = (uint32_t)(p.units % grid);
-    fn<<<grid, kCtsThreads, cts_smem(dir), s>>>(q);
-    return cudaGetLastError();
+    return launch(fn, grid, kCtsThreads, cts_smem(dir), s, q);
 }
 
 // A group (32 whole-page chains, one warp) is one long serial job, so the
@@ -1132,8 +1172,7 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
         auto fn = cbc_enc_split_fn(nr, lanes);
         if (!fn) return cudaErrorInvalidValue;
         const uint64_t teams = (p.npages + 32 / lanes - 1) / (32 / lanes);
-        fn<<<(int)std::min<uint64_t>(teams, sms), kCbcSplitThreads, kSmemEnc, s>>>(p);
-        return cudaGetLastError();
+        return launch(fn, (int)std::min<uint64_t>(teams, sms), kCbcSplitThreads, kSmemEnc, s, p);
     }
     // The tensor tiles take a seventh of the staging traffic off the
     // shared-memory path, which pays once that path is the bound: from 12
@@ -1153,8 +1192,7 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
             std::memcpy(t.rk, p.rk, sizeof(t.rk));
             const int grid = num_sms;
             const int warps = cbc_enc_staged_warps(groups, num_sms);
-            fn<<<grid, warps * 32, kSmemEncTma, s>>>(t);
-            return cudaGetLastError();
+            return launch(fn, grid, warps * 32, kSmemEncTma, s, t);
         }
     }
     if (p.bpp % kStageBlocks == 0) {
@@ -1162,16 +1200,14 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
         if (!fn) return cudaErrorInvalidValue;
         const int grid = (int)(groups < (uint64_t)num_sms ? (groups ? groups : 1) : num_sms);
         const int warps = cbc_enc_staged_warps(groups, num_sms);
-        fn<<<grid, warps * 32, kSmemEnc + warps * kStageWarpSmem, s>>>(p);
-        return cudaGetLastError();
+        return launch(fn, grid, warps * 32, kSmemEnc + warps * kStageWarpSmem, s, p);
     }
     auto fn = cbc_fn(nr, true);
     if (!fn) return cudaErrorInvalidValue;
     // a 32-page group is a heavy work item (32 chains of whole pages): give
     // every SM work as soon as there are as many groups as SMs
     const int grid = (int)(groups < (uint64_t)num_sms ? (groups ? groups : 1) : num_sms);
-    fn<<<grid, kBulkThreads, kSmemEnc, s>>>(p);
-    return cudaGetLastError();
+    return launch(fn, grid, kBulkThreads, kSmemEnc, s, p);
 }
 
 }  // namespace kgpu
