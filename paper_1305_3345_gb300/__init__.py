@@ -131,6 +131,8 @@ def library_path() -> str:
 def lib() -> ctypes.CDLL:
     """The loaded C library (built on first use)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             L = ctypes.CDLL(ensure_built())
@@ -178,7 +180,7 @@ def lib() -> ctypes.CDLL:
                 f = getattr(L, name)
                 f.argtypes = args
                 f.restype = res
-            _lib = L
+            _lib = L  # last: seen without the lock only once it is complete
     return _lib
 
 
@@ -188,9 +190,19 @@ def _check(rc: int, what: str) -> int:
     return rc
 
 
+_torch = None
+
+
+def _import_torch():
+    global _torch
+    import torch
+    _torch = torch
+    return torch
+
+
 def _dev_buf(t):
     """(pointer, nbytes) of a contiguous uint8 CUDA tensor."""
-    import torch
+    torch = _torch or _import_torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("expected a CUDA torch.Tensor")
     if t.dtype != torch.uint8 or not t.is_contiguous():
@@ -216,8 +228,10 @@ def _host_buf(a):
 
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle without a Stream object around it, which
+        # takes 2.9 us of a call's 9.8 (0.3 this way)
+        torch = _torch or _import_torch()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -535,14 +549,34 @@ def kgpu_serve_submit_many(ctx, reqs):
     return rc, tickets[: acc.value]
 
 
+class _PollBuf:
+    """Where kgpu_serve_poll's C call writes a request's status and stamps."""
+
+    def __init__(self):
+        self.status = ctypes.c_int()
+        self.stamps = (ctypes.c_uint64 * 2)()
+        self.args = (ctypes.byref(self.status), self.stamps)
+
+
+# Buffers between polls: making one takes longer than a poll.  A call takes one
+# for itself, so threads and reentrant calls never share; it holds as many as
+# polls have ever run at once.
+_poll_bufs = []
+
+
 def kgpu_serve_poll(ctx, ticket: int, timeout_ns: int = -1):
     """(rc, status, (t_first_tile, t_done)) -- rc 0 when complete, -110 while pending."""
-    st = ctypes.c_int()
-    stamps = (ctypes.c_uint64 * 2)()
-    rc = lib().kgpu_serve_poll(ctx, ticket, timeout_ns, ctypes.byref(st), stamps)
+    try:
+        b = _poll_bufs.pop()
+        b.status.value = b.stamps[0] = b.stamps[1] = 0
+    except IndexError:
+        b = _PollBuf()
+    rc = lib().kgpu_serve_poll(ctx, ticket, timeout_ns, *b.args)
+    out = rc, b.status.value, (b.stamps[0], b.stamps[1])
+    _poll_bufs.append(b)
     if rc not in (0, -110):
         _check(rc, "kgpu_serve_poll")
-    return rc, st.value, (stamps[0], stamps[1])
+    return out
 
 
 def kgpu_serve_stop(ctx, drain_timeout_ns: int = -1) -> int:
