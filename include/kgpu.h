@@ -206,17 +206,21 @@ int kgpu_aes_ecb_crypt(kgpu_ctx *ctx, kgpu_key key, int dir, const void *src, vo
 /*
  * XTS over HOST-resident pages, the paper's pinned-buffer pipeline (section
  * 3.1, "Data Copy Overhead", and the buffer rotation of section 3.2): the
- * buffer is cut into chunk_bytes pieces (a multiple of du_size; 0 = 4 MiB),
- * and each piece is copied host-to-device, transformed and copied back on one
- * of three library-owned streams (one chunk in, one transformed, one out), so
- * copies overlap compute.  src and dst are
- * HOST pointers (pinned memory gives full link speed; pageable memory works
- * but is slower); src == dst is allowed.  Blocks until dst holds the result.
- * Device staging buffers are owned by the context and reused across calls.
+ * buffer is cut into chunk_bytes pieces (a multiple of du_size; 0 = 4 MiB,
+ * unless the pages can be used in place, below), and each piece is copied
+ * host-to-device, transformed and copied back on one of three library-owned
+ * streams (one chunk in, one transformed, one out), so copies overlap compute.
+ * src and dst are HOST pointers (pinned memory gives full link speed; pageable
+ * memory works but is slower); src == dst is allowed.  Blocks until dst holds
+ * the result.  Device staging buffers are owned by the context and reused
+ * across calls.
  * When both [src, src + len) and [dst, dst + len) lie inside ranges
  * registered with kgpu_host_register, there is no staging and no copy: the
  * kernel reads and writes the host pages in place over the host link, and
- * chunk_bytes is ignored.  kgpu_host_unregister waits for such a call.
+ * chunk_bytes is ignored.  kgpu_host_unregister waits for such a call.  With
+ * chunk_bytes 0 the pages are also used in place when each of the two lies
+ * inside one page-locked, mapped allocation or registration known to the CUDA
+ * driver.
  */
 int kgpu_aes_xts_crypt_host(kgpu_ctx *ctx, kgpu_key key, int dir, const void *src, void *dst, size_t len,
                             size_t du_size, uint64_t first_sector, size_t chunk_bytes);

@@ -260,6 +260,37 @@ inline int check_device_range(const kgpu_ctx* ctx, const void* p, size_t len) {
     return KGPU_OK;
 }
 
+// Whether [p, p + len) lies inside one page-locked host allocation or
+// registration that is mapped for the current device; *dev receives the
+// address the device sees for p.  One driver call, made afresh for every
+// request, so nothing is trusted after the caller could have freed it.
+inline bool pinned_range(const void* p, size_t len, uintptr_t* dev) {
+    typedef CUresult (*AttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static AttributesFn fn = []() -> AttributesFn {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return reinterpret_cast<AttributesFn>(f);
+    }();
+    if (!fn || !p) return false;
+    unsigned int type = 0;
+    CUdeviceptr start = 0, mapped = 0;
+    size_t size = 0;
+    CUpointer_attribute which[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                    CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER};
+    void* out[4] = {&type, &start, &size, &mapped};
+    if (fn(4, which, out, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    const uintptr_t a = (uintptr_t)p;
+    if (type != CU_MEMORYTYPE_HOST || !mapped || a < start || a - start > size || len > size - (a - start)) return false;
+    *dev = (uintptr_t)mapped;
+    return true;
+}
+
 inline int check_host_ptr(const void* p) {
     if (!p) return KGPU_EFAULT;
     cudaPointerAttributes a;

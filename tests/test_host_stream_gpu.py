@@ -73,3 +73,32 @@ def test_host_call_on_registered_pages_in_place_over_the_link(ctx, bits, du):
         ctx.host_unregister(dst)
     ctx.delkey(kh)
 
+
+
+@pytest.mark.parametrize("bits,du,units", [(256, 4096, 1), (256, 4096, 2051), (128, 512, 40 * 32 * 4 + 1), (256, 528, 997),
+                                           (128, 48, 5003)])
+def test_host_call_on_pinned_pages_without_a_chunk_size(ctx, bits, du, units):
+    """Pinned buffers that were not registered with the library and no chunk
+    size: used in place over the link, at interior offsets too.  A buffer that
+    is not pinned over its whole length, and an explicit chunk size, take the
+    copy pipeline.  The same bytes each way."""
+    import torch
+    key = w.xts_key(23 + bits, bits)
+    n = du * units
+    data = w.seeded_bytes(23 + du, w.STREAM_DATA, n)
+    ref = oracle.xts(key, 0, data, du, 2**40 + 3)
+    kh = ctx.setkey(key, True)
+    pinned = torch.zeros(2 * n + 64, dtype=torch.uint8).pin_memory()
+    src, dst = pinned[16:16 + n], pinned[n + 48 - n % 16:][:n]
+    src.copy_(torch.from_numpy(data))
+    pageable = np.zeros(n + 16, dtype=np.uint8)
+    pageable = pageable[(-pageable.ctypes.data) % 16:][:n]
+    for out, chunk in ((dst, 0), (dst, 4 << 20), (pageable, 0)):
+        out[:] = 0
+        ctx.xts_crypt_host(kh, 0, src, out, du, 2**40 + 3, chunk)
+        assert np.array_equal(np.asarray(out), ref), (du, units, chunk)
+    assert not pinned[:16].any() and not pinned[n + 16:dst.storage_offset()].any()
+    assert not pinned[dst.storage_offset() + n:].any()
+    ctx.xts_crypt_host(kh, 1, dst, dst, du, 2**40 + 3, 0)   # in place
+    assert np.array_equal(dst.numpy(), data)
+    ctx.delkey(kh)
