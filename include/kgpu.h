@@ -296,7 +296,8 @@ typedef struct kgpu_tuning {
     uint32_t threads;      /* threads per CTA: 512 or 1024 (default 512); a batch holding
                               CBC encryption of host pages runs with 512, the kernel
                               that stages those pages through whole-line copies */
-    uint32_t tile_chunks;  /* work per XTS/ECB tile in 512-byte chunks (default 32 = 16 KiB);
+    uint32_t tile_chunks;  /* work per XTS/ECB tile in 512-byte chunks (default 32 = 16 KiB, less
+                              for a batch that would then have fewer tiles than warps);
                               CBC-decrypt tiles hold the same bytes in whole pages,
                               CBC-encrypt tiles hold up to 32 pages (one chain per lane) */
     uint32_t ctas;         /* CTAs of the persistent kernel (default 0 = one per SM) */

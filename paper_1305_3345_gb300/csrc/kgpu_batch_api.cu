@@ -44,25 +44,18 @@ int tuning_ok(const kgpu_tuning* t) {
 // Validate all requests and pack header | descriptors | tile prefix into buf
 // (which must hold batch_bytes(n)).  Returns the first error, with every
 // request's own code in req_status when given.
-int pack_batch(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, uint32_t tile_chunks, uint64_t warps, uint8_t* buf,
-               int* req_status) {
+int pack_batch(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, uint32_t tile_chunks, uint32_t ctas,
+               uint32_t warps_per_cta, uint8_t* buf, int* req_status) {
     RangeCache rc;
     int first = KGPU_OK;
     ReqDesc* descs = reinterpret_cast<ReqDesc*>(buf + batch_desc_offset());
-    uint64_t* prefix = reinterpret_cast<uint64_t*>(buf + batch_prefix_offset((uint32_t)n));
-    uint32_t* order = reinterpret_cast<uint32_t*>(buf + batch_order_offset((uint32_t)n));
     for (size_t i = 0; i < n; i++) {
         int r = make_desc(ctx, reqs[i], rc, tile_chunks, &descs[i]);
         if (req_status) req_status[i] = r;
         if (r && !first) first = r;
         if (r) descs[i].nblocks = 0;  // refused: no tiles
     }
-    const uint64_t tiles = order_batch(descs, (uint32_t)n, [&](uint32_t i) { return descs[i].nblocks == 0; },
-                                       2 * warps, prefix, order);
-    BatchHeader* h = reinterpret_cast<BatchHeader*>(buf);
-    h->total_tiles = tiles;
-    h->nreq = (uint32_t)n;
-    h->tag = 0;
+    plan_batch(buf, (uint32_t)n, [&](uint32_t i) { return descs[i].nblocks == 0; }, ctas, warps_per_cta);
     return first;
 }
 
@@ -189,7 +182,7 @@ int prepare_slot(kgpu_ctx* ctx, kgpu::BatchSlot& s, size_t n, const kgpu_tuning&
     mp.dst = s.d_counter;
     mp.value = 0;
     mp.elementSize = 4;
-    mp.width = 2;
+    mp.width = 4;  // both work counters
     mp.height = 1;
     ok = ok && cudaGraphAddMemsetNode(&n_ctr, g, nullptr, 0, &mp) == cudaSuccess;
     mp.dst = s.d_status;
@@ -303,6 +296,7 @@ int kgpu_submit(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, kgpu_stream s
     kgpu_tuning t = effective(ctx);
     // CBC encryption of host pages is staged only in the 512-thread kernel
     if (t.threads > 512 && needs_staging(reqs, n)) t.threads = 512;
+    if (!ctx->tune.tile_chunks) t.tile_chunks = default_tile_chunks(reqs, n, (uint64_t)t.ctas * (t.threads / 32));
     const uint64_t ticket = ++ctx->next_ticket;
     kgpu::BatchSlot& s = ctx->slots[ticket % kBatchSlots];
     // a batch someone waits on (kgpu_poll, kgpu_poll_each) keeps its slot
@@ -322,7 +316,7 @@ int kgpu_submit(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, kgpu_stream s
     s.issued = false;
     int rc = prepare_slot(ctx, s, n ? n : 1, t);
     if (rc) return rc;
-    rc = pack_batch(ctx, reqs, n, t.tile_chunks, (uint64_t)t.ctas * (t.threads / 32), s.h_buf, req_status);
+    rc = pack_batch(ctx, reqs, n, t.tile_chunks, t.ctas, t.threads / 32, s.h_buf, req_status);
     if (rc) return rc;
     s.nreq = (uint32_t)n;
     s.gen = ticket;
@@ -480,8 +474,7 @@ int kgpu_autotune(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, kgpu_stream
     for (uint32_t tc : tile_opts) {
         if (rc) break;
         for (uint32_t th : thread_opts) {
-            // the run order's tail reserve depends on the warp count
-            rc = pack_batch(ctx, reqs, n, tc, (uint64_t)ctx->num_sms * (th / 32), hbuf.data(), nullptr);
+            rc = pack_batch(ctx, reqs, n, tc, (uint32_t)ctx->num_sms, th / 32, hbuf.data(), nullptr);
             if (rc) break;
             if (cudaMemcpy(dbuf, hbuf.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
                 rc = KGPU_EIO;

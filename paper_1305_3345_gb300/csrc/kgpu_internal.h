@@ -83,6 +83,9 @@ struct BatchHeader {
     uint64_t total_tiles;
     uint32_t nreq;
     uint32_t tag;  // low 32 bits of the batch's ticket, in its completion words
+    uint64_t long_tiles;  // the CBC-encryption tiles: the first ones in run order
+    uint32_t long_warps;  // warps per CTA that start with them
+    uint32_t pad;
 };
 
 // Byte layout of a batch on the device: header, descriptors, tile prefix, run order.
@@ -106,7 +109,7 @@ struct BatchArgs {
     const DevKey* keys;
     uint32_t max_keys;
     uint32_t scratch_warps;         // warps (by global index) that have a scratch area
-    unsigned long long* next_tile;  // work counter (zero before launch)
+    unsigned long long* next_tile;  // work counters: CBC-encryption tiles, others (zero before launch)
     int* status;                    // per request: 0, or a negative KGPU_E* set by the kernel
     uint4* scratch;                 // kStageWarpBytes per warp, or null
     unsigned long long* fin;        // per request: tiles finished (zero before launch), or null

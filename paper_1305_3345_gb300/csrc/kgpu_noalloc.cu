@@ -120,16 +120,15 @@ extern "C" int kgpu_submit_noalloc(kgpu_ctx* ctx, const kgpu_request* reqs, size
     std::lock_guard<std::mutex> blk(ctx->batch_mu);
     const kgpu_tuning t = ctx->tune;
     uint32_t threads = t.threads ? t.threads : kBatchDefaultThreads;
-    const uint32_t tile_chunks = t.tile_chunks ? t.tile_chunks : kBatchDefaultTileChunks;
     const uint32_t ctas = t.ctas ? t.ctas : (uint32_t)ctx->num_sms;
     // CBC encryption of host pages is staged only in the 512-thread kernel
     if (threads > 512 && needs_staging(reqs, n)) threads = 512;
+    const uint32_t tile_chunks =
+        t.tile_chunks ? t.tile_chunks : default_tile_chunks(reqs, n, (uint64_t)ctas * (threads / 32));
 
     std::lock_guard<std::mutex> lk(g_pack_mu);
     FixedRangeCache cache;
     ReqDesc* descs = reinterpret_cast<ReqDesc*>(g_pack + batch_desc_offset());
-    uint64_t* prefix = reinterpret_cast<uint64_t*>(g_pack + batch_prefix_offset((uint32_t)n));
-    uint32_t* order = reinterpret_cast<uint32_t*>(g_pack + batch_order_offset((uint32_t)n));
     int first = KGPU_OK;
     for (size_t i = 0; i < n; i++) {
         int r = make_desc(ctx, reqs[i], cache, tile_chunks, &descs[i]);
@@ -137,12 +136,7 @@ extern "C" int kgpu_submit_noalloc(kgpu_ctx* ctx, const kgpu_request* reqs, size
         if (r && !first) first = r;
     }
     if (first) return first;
-    const uint64_t tiles = order_batch(descs, (uint32_t)n, [](uint32_t) { return false; },
-                                       2 * (uint64_t)ctas * (threads / 32), prefix, order);
-    BatchHeader* h = reinterpret_cast<BatchHeader*>(g_pack);
-    h->total_tiles = tiles;
-    h->nreq = (uint32_t)n;
-    h->tag = 0;
+    plan_batch(g_pack, (uint32_t)n, [](uint32_t) { return false; }, ctas, threads / 32);
 
     BatchArgs a{};
     a.buf = scratch + kBatchOff;

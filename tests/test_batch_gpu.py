@@ -379,3 +379,27 @@ def test_concurrent_submitters_share_the_slots(ctx):
     assert ctx.poll(ctx.submit(r), -1) == 0
     assert np.array_equal(outs[0][:8192].cpu().numpy(), oracle.xts(key, 0, data[:8192], 4096, 0))
     ctx.delkey(kh)
+
+
+@pytest.mark.parametrize("n,modes,lo,hi,unit,threads,ctas", [
+    (1, (0.0, 0.0), 4096, 4096, 4096, 512, 0),            # one CBC-encryption tile, no other
+    (40, (0.0, 0.0), 4096, 1 << 20, 4096, 512, 0),        # CBC encryption alone: one queue empty
+    (40, (0.6, 0.4), 4096, 65536, 4096, 512, 0),          # none: the other queue empty
+    (60, (0.2, 0.1), 4096, 1 << 20, 4096, 512, 0),        # mostly CBC encryption
+    (300, (0.5, 0.4), 4096, 131072, 4096, 1024, 0),       # the 1,024-thread kernel
+    (90, (0.4, 0.2), 4096, 262144, 512, 512, 3),          # few CTAs: many rounds of either queue
+    (90, (0.4, 0.2), 4096, 65536, 64, 512, 700),          # more CTAs than run at once
+])
+def test_batch_queues(ctx, n, modes, lo, hi, unit, threads, ctas):
+    """CBC encryption and everything else have a queue each; the share of
+    either, the launch shape and the tile size the library picks (none is set)
+    do not change a byte."""
+    ctx.set_tuning(threads, 0, ctas)
+    try:
+        b = Batch(ctx, 71 + n, n, lo, hi, 6, unit=unit, modes=(*modes, 1.0 - sum(modes)), ecb=0.0)
+        run(ctx, b.reqs)
+        for i in range(n):
+            assert np.array_equal(b.got(i), b.expected(i)), (i, int(b.modes[i]), int(b.sizes[i]))
+        b.close()
+    finally:
+        ctx.set_tuning(0, 0, 0)
