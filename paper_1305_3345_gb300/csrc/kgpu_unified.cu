@@ -453,33 +453,42 @@ __device__ __forceinline__ void tile_cbc_enc(const ReqDesc& d, uint64_t p0, uint
 // warp -- the form for a lightly loaded device, where a request's latency is
 // its chain time.  Each round a lane fetches the three other columns of its
 // state from its quad (three independent shuffles), looks up its own column
-// (the two-table round of uni_col) and reads its own round-key word from the
-// warp's key slot (the quad's four words share one wavefront).  Lanes without
-// a page step along with predicated-off memory accesses.
+// (the two-table round of uni_col) and takes its own round-key word from a
+// register.  Lanes without a page step along with predicated-off memory
+// accesses.
+
+// A quad lane's round-key words: its column of every round, read from the
+// warp's key slot once per tile (64 served CBC-encryption requests, 12 MB: 275
+// us with a shared load every round, 251 this way).
+template <int NR>
+struct QuadKeys {
+    uint32_t k[NR + 1];
+    __device__ __forceinline__ explicit QuadKeys(uint32_t key) {  // key: shared address of its column of round 0
+#pragma unroll
+        for (int r = 0; r <= NR; r++)
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(k[r]) : "r"(key + 16u * (r < NR ? r : 14)));
+    }
+};
+
 // One block of a four-lane chain: x is this lane's column of the block to
-// encipher (plaintext xor chain value), key the shared address of its column
-// of round 0 (words 4r + col of the schedule).
+// encipher (plaintext xor chain value).  The columns of the rotated half of
+// the round are asked for first, so that the rotation waits for nothing else.
 template <int NR>
 __device__ __forceinline__ uint32_t quad_encrypt(uint32_t x, uint32_t s1, uint32_t s2, uint32_t s3,
-                                                 const UniLanes& L, uint32_t key) {
-    auto key_word = [&](int r) {
-        uint32_t v;
-        asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(key + 16u * (uint32_t)r));
-        return v;
-    };
-    x ^= key_word(0);
+                                                 const UniLanes& L, const QuadKeys<NR>& K) {
+    x ^= K.k[0];
 #pragma unroll
     for (int r = 1; r < NR; r++) {
-        const uint32_t a1 = __shfl_sync(0xffffffffu, x, s1);
         const uint32_t a2 = __shfl_sync(0xffffffffu, x, s2);
         const uint32_t a3 = __shfl_sync(0xffffffffu, x, s3);
-        x = uni_col(x, a1, a2, a3, key_word(r), L);
+        const uint32_t a1 = __shfl_sync(0xffffffffu, x, s1);
+        x = uni_col(x, a1, a2, a3, K.k[r], L);
     }
     const uint32_t a1 = __shfl_sync(0xffffffffu, x, s1);
     const uint32_t a2 = __shfl_sync(0xffffffffu, x, s2);
     const uint32_t a3 = __shfl_sync(0xffffffffu, x, s3);
 #define KGPU_FIN(P, v) lds_tab<kSmemBase>(row_addr<P>(v, L.f))
-    return merge_bytes(KGPU_FIN(0, x), KGPU_FIN(1, a1), KGPU_FIN(2, a2), KGPU_FIN(3, a3)) ^ key_word(14);
+    return merge_bytes(KGPU_FIN(0, x), KGPU_FIN(1, a1), KGPU_FIN(2, a2), KGPU_FIN(3, a3)) ^ K.k[NR];
 #undef KGPU_FIN
 }
 
@@ -493,7 +502,7 @@ __device__ __forceinline__ void quad_chains(const ReqDesc& d, uint64_t p0, uint6
     const uint32_t bpp = d.unit_blocks;
     const uint32_t* in = reinterpret_cast<const uint32_t*>(d.src + (valid ? page : p0) * bpp) + c;
     uint32_t* out = reinterpret_cast<uint32_t*>(d.dst + (valid ? page : p0) * bpp) + c;
-    const uint32_t key = K.data_saddr + 4u * c;  // word 4r + c of the schedule: round r, this column
+    const QuadKeys<NR> key(K.data_saddr + 4u * c);  // word 4r + c of the schedule: round r, this column
     const uint32_t s1 = base | ((c + 1) & 3u), s2 = base | ((c + 2) & 3u), s3 = base | ((c + 3) & 3u);
     uint32_t x = valid ? reinterpret_cast<const uint32_t*>(d.ivs + page)[c] : 0u;
     // the chain is sequential, so plaintext is fetched four blocks ahead
@@ -549,7 +558,7 @@ __device__ __forceinline__ void quad_chains_staged(const ReqDesc& d, uint64_t p0
     const UniLanes L = uni_lanes(lane, 0);
     const bool valid = p0 + qp < p1;
     const uint32_t bpp = d.unit_blocks;
-    const uint32_t key = K.data_saddr + 4u * c;
+    const QuadKeys<NR> key(K.data_saddr + 4u * c);
     const uint32_t s1 = base | ((c + 1) & 3u), s2 = base | ((c + 2) & 3u), s3 = base | ((c + 3) & 3u);
     uint32_t x = valid ? reinterpret_cast<const uint32_t*>(d.ivs + p0 + qp)[c] : 0u;
     // copy positions: lanes 8p..8p+7 move page p's line (pages 0-3, then 4-7)
