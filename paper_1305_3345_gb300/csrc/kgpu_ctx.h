@@ -85,6 +85,8 @@ struct ServeState {
     uint32_t nslots = 0;
     uint64_t tile_ring = 0;  // entries of the device tile ring
     uint32_t tile_chunks = 8;
+    bool auto_tiles = false;  // no tile size configured: bursts may take larger ones
+    uint32_t workers = 0;     // worker warps of the kernel
     uint64_t admit_bytes = 0;
     uint64_t next_seq = 0;
     uint64_t inflight_bytes = 0;

@@ -75,6 +75,8 @@ int serve_alloc(kgpu_ctx* ctx, ServeState& st, const kgpu_serve_config* cfg) {
     // switches to 32-KiB tiles
     st.tile_chunks = c.tile_chunks ? c.tile_chunks : 2;
     if (st.tile_chunks > (1u << 20)) return KGPU_EINVAL;
+    st.auto_tiles = !c.tile_chunks;
+    st.workers = (uint32_t)ctx->num_sms * (kServeThreads / 32) - 1;
     st.admit_bytes = c.admit_bytes ? c.admit_bytes : ctx->cfg.admit_bytes;
     const uint64_t idle = c.idle_timeout_ns ? c.idle_timeout_ns : ctx->cfg.idle_timeout_ns;
     const uint64_t life = c.lifetime_ns ? c.lifetime_ns : 30000000000ull;
@@ -289,8 +291,17 @@ bool backlogged(const ServeState& st) {
     return load_acquire(&st.done_seq[seq & (st.nslots - 1)]) < seq + 1;
 }
 
-int stage(ServeState& st, const ReqDesc& dreq, uint64_t* seq_out) {
+// Requests that arrive together are a small backlog of their own: a burst of
+// burst_bytes gets tiles that leave every worker warp at least four, between
+// the default size and the backlog's, unless the caller set a size (a burst of
+// 128 XTS requests, 24 MB: 130 us in 1-KiB tiles, 112 in 2-KiB ones).
+int stage(ServeState& st, const ReqDesc& dreq, uint64_t burst_bytes, uint64_t* seq_out) {
     ReqDesc d = dreq;
+    if (st.auto_tiles && d.mode != KGPU_MODE_COPY) {
+        uint32_t t = st.tile_chunks;
+        while (t < kBacklogTileChunks && burst_bytes / (512ull * 8 * t) >= st.workers) t *= 2;
+        set_tile_units(d, t);
+    }
     if (backlogged(st)) {
         set_tile_units(d, std::max<uint32_t>(st.tile_chunks, kBacklogTileChunks));
     } else if (d.mode == KGPU_MODE_CBC_ENC &&
@@ -353,7 +364,7 @@ int commit(kgpu_ctx* ctx, ServeState& st) {
 }
 
 int publish(kgpu_ctx* ctx, ServeState& st, const ReqDesc& d, uint64_t* seq_out) {
-    int r = stage(st, d, seq_out);
+    int r = stage(st, d, d.nblocks * 16, seq_out);
     return r ? r : commit(ctx, st);
 }
 
@@ -562,9 +573,11 @@ int kgpu_serve_submit_many(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, kg
     }
     size_t k = 0;
     int r = KGPU_OK;
+    uint64_t burst = 0;
+    for (size_t i = 0; i < n; i++) burst += reqs[i].len;
     for (; k < n; k++) {
         uint64_t seq = 0;
-        if ((r = stage(st, descs[k], &seq))) break;
+        if ((r = stage(st, descs[k], burst, &seq))) break;
         tickets[k] = seq + 1;
     }
     *accepted = k;
@@ -838,9 +851,11 @@ static int replay_serve_impl(kgpu_ctx* ctx, const kgpu_request* reqs, const uint
         {
             std::lock_guard<std::mutex> lk(ctx->serve_mu);
             const uint64_t t = now_ns();
+            uint64_t burst = 0;
+            for (size_t q = i; q < n && q - i < 256 && t0 + arrival_ns[q] <= t; q++) burst += reqs[q].len;
             for (; j < n && j - i < 256 && t0 + arrival_ns[j] <= t; j++) {
                 uint64_t seq = 0;
-                r = stage(st, descs[j], &seq);
+                r = stage(st, descs[j], burst, &seq);
                 if (r) break;
                 if (detail) detail[3 * j] = t - (t0 + arrival_ns[j]);
                 seq_of[j].store(seq, std::memory_order_release);
