@@ -61,6 +61,9 @@ constexpr uint32_t kDescSrcHost = 1u;  // source in registered host memory
 constexpr uint32_t kDescDstHost = 2u;  // destination in registered host memory
 constexpr uint32_t kDescQuad = 4u;     // CBC encryption, four lanes per page: tiles of kQuadPages pages
 constexpr uint32_t kQuadPages = 8;
+constexpr uint32_t kDescSplit = 8u;    // CBC encryption, two lanes per page: tiles of kSplitPages pages
+constexpr uint32_t kSplitPages = 16;
+constexpr int kSplitThreads = 512;     // the batch-kernel variant that has the registers for it
 
 // Per-warp device scratch of the unified kernels: CBC encryption of
 // host-resident pages moves 8 blocks of each of a warp's 32 pages through it

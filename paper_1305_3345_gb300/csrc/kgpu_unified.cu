@@ -416,6 +416,105 @@ __device__ __forceinline__ void tile_cbc_dec(const ReqDesc& d, uint64_t p0, uint
     }
 }
 
+// CBC encryption of pages [p0, p1), at most 16, two lanes per page: lane 2q + c
+// holds columns 2c and 2c + 1 of page q's chain state.  Each round a lane takes
+// the other two columns from its neighbour by shuffle and looks up its own two
+// columns: about 100 cycles a round, against 150 with a lane per page.  The
+// round keys sit in registers and the rounds are unrolled, with exits for the
+// shorter keys, so that one body serves every key size.
+struct PairKeys {
+    uint2 first, last, mid[13];
+    int nr;
+    __device__ __forceinline__ PairKeys(const WarpKeys& K, uint32_t c) : nr(K.nr) {
+        auto load = [&](uint32_t r) {
+            uint2 v;
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(K.data_saddr + 8u * c + 16u * r));
+            return v;
+        };
+        first = load(0);
+        last = load(14);
+#pragma unroll
+        for (uint32_t r = 1; r <= 13; r++) mid[r - 1] = load(r);  // those from nr on are not used
+    }
+};
+
+__device__ __forceinline__ void pair_round(uint32_t& x0, uint32_t& x1, const uint2& k, const UniLanes& L) {
+    const uint32_t y0 = __shfl_xor_sync(0xffffffffu, x0, 1);
+    const uint32_t y1 = __shfl_xor_sync(0xffffffffu, x1, 1);
+    // the own columns' lookups go out while the shuffles are on their way
+    const uint32_t a0 = lds_tab<kSmemBase>(row_addr<0>(x0, L.r0)), b0 = lds_tab<kSmemBase>(row_addr<1>(x1, L.r1));
+    const uint32_t a1 = lds_tab<kSmemBase>(row_addr<0>(x1, L.r0)), d1 = lds_tab<kSmemBase>(row_addr<3>(x0, L.r1));
+    const uint32_t c0 = lds_tab<kSmemBase>(row_addr<2>(y0, L.r0)), d0 = lds_tab<kSmemBase>(row_addr<3>(y1, L.r1));
+    const uint32_t c1 = lds_tab<kSmemBase>(row_addr<2>(y1, L.r0)), b1 = lds_tab<kSmemBase>(row_addr<1>(y0, L.r1));
+    x0 = a0 ^ b0 ^ rotl16(c0 ^ d0 ^ k.x);
+    x1 = a1 ^ b1 ^ rotl16(c1 ^ d1 ^ k.y);
+}
+
+__device__ __forceinline__ void pair_encrypt(uint32_t& x0, uint32_t& x1, const PairKeys& k, const UniLanes& L) {
+    x0 ^= k.first.x;
+    x1 ^= k.first.y;
+#pragma unroll
+    for (int r = 1; r <= 9; r++) pair_round(x0, x1, k.mid[r - 1], L);
+    if (k.nr > 10) {
+        pair_round(x0, x1, k.mid[9], L);
+        pair_round(x0, x1, k.mid[10], L);
+        if (k.nr > 12) {
+            pair_round(x0, x1, k.mid[11], L);
+            pair_round(x0, x1, k.mid[12], L);
+        }
+    }
+    const uint32_t y0 = __shfl_xor_sync(0xffffffffu, x0, 1);
+    const uint32_t y1 = __shfl_xor_sync(0xffffffffu, x1, 1);
+#define KGPU_FIN(P, v) lds_tab<kSmemBase>(row_addr<P>(v, L.f))
+    const uint32_t o0 = merge_bytes(KGPU_FIN(0, x0), KGPU_FIN(1, x1), KGPU_FIN(2, y0), KGPU_FIN(3, y1)) ^ k.last.x;
+    const uint32_t o1 = merge_bytes(KGPU_FIN(0, x1), KGPU_FIN(1, y0), KGPU_FIN(2, y1), KGPU_FIN(3, x0)) ^ k.last.y;
+#undef KGPU_FIN
+    x0 = o0;
+    x1 = o1;
+}
+
+__device__ __forceinline__ void tile_cbc_enc_pair(const ReqDesc& d, uint64_t p0, uint64_t p1, const WarpKeys& K) {
+    __syncwarp();
+    const uint32_t lane = lane_id(), c = lane & 1u;
+    const UniLanes L = uni_lanes(lane, 0);
+    const PairKeys key(K, c);
+    const uint32_t bpp = d.unit_blocks;
+    const uint4 z = make_uint4(0, 0, 0, 0);
+    // lanes without a page step along, loads and stores predicated off
+    const uint64_t page = p0 + (lane >> 1);
+    const bool valid = page < p1;
+    const uint4* in = d.src + (valid ? page : p0) * bpp;
+    uint4* out = d.dst + (valid ? page : p0) * bpp;
+    uint2 x = valid ? reinterpret_cast<const uint2*>(d.ivs + page)[c] : make_uint2(0, 0);
+    // a lane moves whole blocks, every other one of its page, and trades halves
+    // with its neighbour; two steps of two blocks are on their way while one is
+    // enciphered
+    uint4 n0 = valid && c < bpp ? in[c] : z;
+    uint4 n1 = valid && c + 2 < bpp ? in[c + 2] : z;
+    uint32_t i = c;
+    for (uint32_t step = 0; step < bpp / 2 + (bpp & 1u); ++step, i += 2) {
+        const uint4 v = n0;
+        n0 = n1;
+        n1 = valid && i + 4 < bpp ? in[i + 4] : z;
+        uint2 give = c ? make_uint2(v.x, v.y) : make_uint2(v.z, v.w);
+        const uint2 keep = c ? make_uint2(v.z, v.w) : make_uint2(v.x, v.y);
+        uint2 got = make_uint2(__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1));
+        uint2 first = make_uint2(0, 0);
+#pragma unroll 1
+        for (uint32_t h = 0; h < 2; h++) {  // the even block, then the odd one
+            const uint2 t = h == c ? keep : got;
+            x.x ^= t.x;
+            x.y ^= t.y;
+            pair_encrypt(x.x, x.y, key, L);
+            if (h == 0) first = x;
+        }
+        // lane 0 stores the even block, lane 1 the odd one
+        give = c ? first : x;
+        got = make_uint2(__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1));
+        if (valid && i < bpp) out[i] = c ? make_uint4(got.x, got.y, x.x, x.y) : make_uint4(first.x, first.y, got.x, got.y);
+    }
+}
+
 // CBC encryption of pages [p0, p1), p1 - p0 <= 32: one chain per lane.
 // Lanes without a page keep stepping with the others (their loads and stores
 // are predicated off), so the warp runs every chain in one converged pass.
@@ -846,6 +945,8 @@ __device__ __forceinline__ int run_tile(const ReqDesc& d, uint64_t tile_in_req, 
                 if (QUAD && (d.flags & kDescQuad) && K.stage_saddr)
                     tile_cbc_enc_quad_staged(d, u0, u1, K, K.stage_saddr);
                 else tile_cbc_enc_staged(d, u0, u1, K, stage);
+            } else if (!QUAD && TWO && (d.flags & kDescSplit)) {
+                tile_cbc_enc_pair(d, u0, u1, K);
             } else if (QUAD && (d.flags & kDescQuad)) {
                 tile_cbc_enc_quad(d, u0, u1, K);
             } else if (pool && !(d.flags & (kDescSrcHost | kDescDstHost)) && d.unit_blocks % kPoolBlocks == 0) {

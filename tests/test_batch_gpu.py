@@ -403,3 +403,45 @@ def test_batch_queues(ctx, n, modes, lo, hi, unit, threads, ctas):
         b.close()
     finally:
         ctx.set_tuning(0, 0, 0)
+
+
+@pytest.mark.parametrize("unit", [16, 32, 48, 128, 4112])
+def test_batch_cbc_encrypt_two_lanes_per_page(ctx, unit):
+    """A batch with few CBC-encryption pages runs two lanes per page: odd and
+    even page lengths, ragged teams, all key sizes, out of place and in place,
+    beside other requests."""
+    import torch
+    import paper_1305_3345_gb300 as kg
+    counts = [1, 2, 15, 16, 17, 33, 100]
+    bits = [128, 192, 256]
+    n = len(counts) * len(bits) * 2
+    pages = [counts[i % len(counts)] for i in range(n)]
+    off = np.concatenate([[0], np.cumsum(np.array(pages) * unit)]).astype(np.int64)
+    ivo = np.concatenate([[0], np.cumsum(pages)]).astype(np.int64)
+    data = w.seeded_bytes(81 + unit, w.STREAM_DATA, int(off[-1]))
+    ivs = w.page_ivs(81 + unit, int(ivo[-1]))
+    src, iv = torch.from_numpy(data.copy()).cuda(), torch.from_numpy(ivs.reshape(-1).copy()).cuda()
+    dst = torch.zeros_like(src)
+    keys = [w.single_key(81, b) for b in bits]
+    h = [ctx.setkey(k, False) for k in keys]
+    r = np.zeros(n + 4, dtype=kg.request_dtype())
+    for i in range(n):
+        out = src if i >= n // 2 else dst
+        r[i]["mode"], r[i]["key"] = kg.MODE_CBC_ENC, h[i % len(bits)]
+        r[i]["src"], r[i]["dst"] = src.data_ptr() + int(off[i]), out.data_ptr() + int(off[i])
+        r[i]["len"], r[i]["unit_size"], r[i]["ivs"] = pages[i] * unit, unit, iv.data_ptr() + 16 * int(ivo[i])
+    other = torch.from_numpy(w.seeded_bytes(82, w.STREAM_DATA, 4 * 65536).copy()).cuda()
+    got_other = torch.zeros_like(other)
+    for i in range(4):
+        r[n + i]["mode"], r[n + i]["key"], r[n + i]["len"] = kg.MODE_ECB, h[i % 3], 65536
+        r[n + i]["src"], r[n + i]["dst"] = other.data_ptr() + i * 65536, got_other.data_ptr() + i * 65536
+    run(ctx, r)
+    a, b = dst.cpu().numpy(), src.cpu().numpy()
+    for i in range(n):
+        ref = oracle.cbc(keys[i % len(bits)], 0, data[off[i]:off[i + 1]], unit, ivs[ivo[i]:ivo[i + 1]])
+        assert np.array_equal((b if i >= n // 2 else a)[off[i]:off[i + 1]], ref), (unit, i, pages[i])
+    for i in range(4):
+        x = other[i * 65536:(i + 1) * 65536].cpu().numpy()
+        assert np.array_equal(got_other[i * 65536:(i + 1) * 65536].cpu().numpy(), oracle.ecb(keys[i % 3], 0, x))
+    for x in h:
+        ctx.delkey(x)
