@@ -312,7 +312,7 @@ typedef struct kgpu_tuning {
  * when req_status is non-NULL, req_status[i] holds each request's own code.
  * The descriptors are copied into one of four rotating pinned staging slots
  * (the paper's four static pinned buffers, section 3.2) and the submission is
- * replayed as a CUDA graph {copy in, clear, kernel, copy status out}.  When
+ * replayed as a CUDA graph {copy in, kernel}.  When
  * all four slots hold unfinished batches, submit blocks until the oldest ends;
  * when the slot it would reuse is being waited on by a kgpu_poll or
  * kgpu_poll_each call, it returns KGPU_EBUSY (retry).  Reusing a slot does not

@@ -18,32 +18,27 @@ namespace kgpu {
 
 // One slot of the batch ring (kgpu_submit): the paper's statically allocated,
 // rotating pinned buffers (section 3.2), here four of them.  Each slot owns its
-// pinned staging area, its device copy, a status array and an instantiated
-// CUDA graph {copy in, reset counter and status, persistent kernel, copy
-// status out}.
+// pinned staging area, its device copy and an instantiated CUDA graph {copy in,
+// persistent kernel}: the counters start at zero because their zeros come with
+// the copy, and the statuses come back in the completion words.
 struct BatchSlot {
     uint64_t gen = 0;            // generation of the last ticket issued on this slot
     bool issued = false;
     cudaEvent_t done = nullptr;  // recorded after the graph
-    uint8_t* h_buf = nullptr;    // pinned: header | descriptors | tile prefix
+    uint8_t* h_buf = nullptr;    // pinned: header | descriptors | tile prefix | run order | zeros
     uint8_t* d_buf = nullptr;
     size_t cap = 0;              // bytes of h_buf / d_buf
-    int* d_status = nullptr;
-    int* h_status = nullptr;     // pinned
-    size_t status_cap = 0;       // entries
-    unsigned long long* d_fin = nullptr;   // per request: tiles finished
+    size_t done_cap = 0;                   // entries of h_done
     unsigned long long* h_done = nullptr;  // pinned, mapped: per-request completion words
     unsigned long long* d_done = nullptr;  // the device's view of h_done
     uint32_t tag = 0;                      // completion tag of the slot's current batch
     int pollers = 0;                       // kgpu_poll / kgpu_poll_each calls holding the slot
-    unsigned long long* d_counter = nullptr;
     uint4* d_scratch = nullptr;  // per-warp staging for CBC encryption of host pages
     uint32_t scratch_warps = 0;
     uint32_t nreq = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    cudaGraphNode_t n_copy = nullptr, n_status_clear = nullptr, n_fin_clear = nullptr, n_kernel = nullptr,
-                    n_status_out = nullptr;
+    cudaGraphNode_t n_copy = nullptr, n_kernel = nullptr;
     int graph_threads = 0, graph_grid = 0;
     BatchArgs args{};
 };

@@ -105,14 +105,23 @@ __host__ __device__ constexpr size_t batch_bytes(uint32_t nreq) {
     return batch_order_offset(nreq) + ((size_t)nreq * sizeof(uint32_t) + 7) / 8 * 8;
 }
 
+// The words a batch starts with at zero may follow the run order, and come with
+// it in one copy: the two work counters, the finished tiles per request, the
+// status per request.
+__host__ __device__ constexpr size_t batch_zeros_offset(uint32_t nreq) { return (batch_bytes(nreq) + 15) / 16 * 16; }
+__host__ __device__ constexpr size_t batch_bytes_with_zeros(uint32_t nreq) {
+    return batch_zeros_offset(nreq) + 16 + (size_t)nreq * (sizeof(unsigned long long) + sizeof(int));
+}
+
 // Arguments of the unified batch kernel (fixed per staging slot, so a captured
 // graph never needs new kernel parameters; the request count is in the header).
 struct BatchArgs {
-    const uint8_t* buf;  // BatchHeader | ReqDesc[nreq] | uint64_t tile_start[nreq + 1]
+    uint8_t* buf;  // BatchHeader | ReqDesc[nreq] | uint64_t tile_start[nreq + 1] | order | zeros if next_tile is null
     const DevKey* keys;
     uint32_t max_keys;
     uint32_t scratch_warps;         // warps (by global index) that have a scratch area
-    unsigned long long* next_tile;  // work counters: CBC-encryption tiles, others (zero before launch)
+    unsigned long long* next_tile;  // work counters: CBC-encryption tiles, others (zero before
+                                    // launch); null: they, fin and status are the zeros in buf
     int* status;                    // per request: 0, or a negative KGPU_E* set by the kernel
     uint4* scratch;                 // kStageWarpBytes per warp, or null
     unsigned long long* fin;        // per request: tiles finished (zero before launch), or null

@@ -1031,6 +1031,14 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
     const ReqDesc* reqs = reinterpret_cast<const ReqDesc*>(a.buf + batch_desc_offset());
     const uint64_t* tile_start = reinterpret_cast<const uint64_t*>(a.buf + batch_prefix_offset(nreq));
     const uint32_t* order = reinterpret_cast<const uint32_t*>(a.buf + batch_order_offset(nreq));
+    unsigned long long* work = a.next_tile;
+    unsigned long long* fin = a.fin;
+    int* status = a.status;
+    if (!work) {
+        work = reinterpret_cast<unsigned long long*>(a.buf + batch_zeros_offset(nreq));
+        fin = work + 2;
+        status = reinterpret_cast<int*>(fin + nreq);
+    }
     // Two queues: the CBC-encryption tiles, whose time is a chain's latency,
     // and the others.  The first long_warps warps of every CTA start with the
     // chains, so that these run beside each other and beside other work from
@@ -1051,41 +1059,41 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
     }
     bool other = true;  // the other queue has not been tried
     unsigned long long next = 0;
-    if (lane == 0) next = atomicAdd(&a.next_tile[on_long ? 0 : 1], 1ull);
+    if (lane == 0) next = atomicAdd(&work[on_long ? 0 : 1], 1ull);
     next = __shfl_sync(0xffffffffu, next, 0);
     for (;;) {
         if (next >= (on_long ? longs : shorts)) {
             if (!other) break;
             other = false;
             on_long = !on_long;
-            if (lane == 0) next = atomicAdd(&a.next_tile[on_long ? 0 : 1], 1ull);
+            if (lane == 0) next = atomicAdd(&work[on_long ? 0 : 1], 1ull);
             next = __shfl_sync(0xffffffffu, next, 0);
             continue;
         }
         const uint64_t t = on_long ? next : longs + next;
         const bool ahead = !on_long && next + 2 * (uint64_t)total_warps() < shorts;
-        if (ahead && lane == 0) next = atomicAdd(&a.next_tile[1], 1ull);
+        if (ahead && lane == 0) next = atomicAdd(&work[1], 1ull);
         const uint32_t k = find_request(tile_start, nreq, t);
         const uint32_t i = order[k];
         const ReqDesc d = reqs[i];
         const int st = run_tile<false, (THREADS <= 512)>(d, t - tile_start[k], a.keys, a.max_keys, K, cur_sel, cur_gen, stage,
                                                            pool);
-        if (st && lane == 0) a.status[i] = st;
-        if (a.fin) {
+        if (st && lane == 0) status[i] = st;
+        if (fin) {
             // per-request completion: the warp that finishes a request's last
             // tile publishes (tag << 32 | status) to the host-mapped word,
             // after an acq_rel count that orders every warp's tile writes
             // before it (the same protocol as the serving ring)
             __syncwarp();
             unsigned long long f = 0;
-            if (lane == 0) f = atom_add_acq_rel_gpu(&a.fin[i], 1ull) + 1;
+            if (lane == 0) f = atom_add_acq_rel_gpu(&fin[i], 1ull) + 1;
             f = __shfl_sync(0xffffffffu, f, 0);
             if (lane == 0 && f == tile_start[k + 1] - tile_start[k]) {
-                const unsigned int code = (unsigned int)*reinterpret_cast<volatile int*>(&a.status[i]);
+                const unsigned int code = (unsigned int)*reinterpret_cast<volatile int*>(&status[i]);
                 st_release_sys(&a.done[i], (unsigned long long)hdr->tag << 32 | code);
             }
         }
-        if (!ahead && lane == 0) next = atomicAdd(&a.next_tile[on_long ? 0 : 1], 1ull);
+        if (!ahead && lane == 0) next = atomicAdd(&work[on_long ? 0 : 1], 1ull);
         next = __shfl_sync(0xffffffffu, next, 0);
     }
 }
