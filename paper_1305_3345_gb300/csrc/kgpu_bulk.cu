@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kCbcSplitThreads, 1) cbc_enc_split_kernel(cons
     using Piece = std::conditional_t<kCols == 1, uint32_t, uint2>;
     const uint32_t lane = lane_id();
     const uint32_t c = lane & (LANES - 1u), team = lane & ~(LANES - 1u);
-    const Rep4 T{lane * 4u, lane * 4u + 128u};
+    const Rep4Permute T{lane * 4u, lane * 4u + 128u};
     uint32_t k[NR + 1][kCols];
 #pragma unroll
     for (int r = 0; r <= NR; r++)
