@@ -497,6 +497,7 @@ int kgpu_aes_xts_crypt_host(kgpu_ctx* ctx, kgpu_key key, int dir, const void* sr
         BulkParams p;
         fill_bulk(&p, k, dir, reinterpret_cast<const void*>(hsrc), reinterpret_cast<void*>(hdst), len, du_size,
                   first_sector);
+        p.link = 1;
         cudaError_t e = launch_xts(p, k.nr, dir, link_sms(ctx, p), ctx->hs[0]);
         cudaError_t e2 = cudaStreamSynchronize(ctx->hs[0]);
         return from_cuda(e != cudaSuccess ? e : e2);

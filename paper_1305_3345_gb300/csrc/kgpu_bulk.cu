@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "aes_device.cuh"
+#include "bitslice_device.cuh"
 #include "kgpu_bulk.h"
 
 namespace kgpu {
@@ -112,28 +113,18 @@ __device__ __forceinline__ uint64_t div_small(uint64_t a, uint32_t b) {
 // 1 MiB of 4-KiB units, AES-256 decryption, back to back on the GPU: 14.4 -> 8.2 us;
 // 16 MiB of encryption 34.9 -> 30.8 us.
 // ---------------------------------------------------------------------------
-template <int NR, int DIR, bool TWEAK>
-__global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_constant__ BulkParams p) {
-    extern __shared__ __align__(128) char smem[];
-    if (!smem_layout_ok(smem)) return;  // uniform over the CTA; refused at init
-    next_may_start();
-    if (DIR == 0) fill_enc(smem);
-    else fill_dec<TWEAK>(smem);
-    wait_for_previous();
-    __syncthreads();
-
+template <int NR, int DIR, bool TWEAK, int WARPS>
+__device__ __forceinline__ void bulk_chunks(const BulkParams& p, uint4* tweaks, uint64_t first, uint32_t own) {
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
-    constexpr uint32_t kWarps = kBulkThreads / 32;
+    constexpr uint32_t kWarps = WARPS;
     const Rep4 T{lane * 4u, lane * 4u + 128u};
     const Rep1<2> IS{lane * 4u};
     const Rep1<2> TE{lane * 4u + 128u};
     const ParamKey K{p.rk};
     const ParamKey TK{p.tk};
 
-    // this CTA's chunks, and this warp's part of them
-    const uint32_t own = p.cta_chunks + (blockIdx.x < p.cta_rest ? 1u : 0u);
-    const uint64_t first = (uint64_t)p.cta_chunks * blockIdx.x + min(blockIdx.x, p.cta_rest);
+    // this warp's part of the run
     const uint32_t wa = (uint32_t)((uint64_t)own * warp / kWarps);
     const uint32_t we = (uint32_t)((uint64_t)own * (warp + 1) / kWarps);
 
@@ -153,12 +144,13 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_cons
 
     const uint32_t bps = p.bps;
     const bool shared = bps >= 32;  // the CTA forms the tweaks together
-    const uint32_t gthreads = shared ? (uint32_t)kBulkThreads : 32u;
+    const uint32_t gthreads = shared ? kWarps * 32u : 32u;
     const uint32_t gwarp = shared ? warp : 0u, gwarps = shared ? kWarps : 1u;
-    uint4* tw = reinterpret_cast<uint4*>(smem + (DIR == 0 ? kSmemEnc : kSmemDec)) + (shared ? 0u : warp * 32u);
+    uint4* tw = tweaks + (shared ? 0u : warp * 32u);
     auto group_sync = [&]() {
-        if (shared) __syncthreads();
-        else __syncwarp();
+        if (!shared) __syncwarp();
+        else if (WARPS * 32 == kBulkThreads) __syncthreads();
+        else asm volatile("bar.sync 1, %0;" ::"n"(WARPS * 32) : "memory");  // the mixed kernel's table warps
     };
     uint64_t c = first + (shared ? 0u : wa);
     uint32_t left = shared ? own : we - wa;
@@ -214,6 +206,141 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_cons
         }
         c += n;
         left -= n;
+    }
+}
+
+// This CTA's run of 32-block chunks.
+__device__ __forceinline__ uint64_t cta_first(const BulkParams& p) {
+    return (uint64_t)p.cta_chunks * blockIdx.x + min(blockIdx.x, p.cta_rest);
+}
+__device__ __forceinline__ uint32_t cta_own(const BulkParams& p) {
+    return p.cta_chunks + (blockIdx.x < p.cta_rest ? 1u : 0u);
+}
+
+template <int NR, int DIR, bool TWEAK>
+__global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_constant__ BulkParams p) {
+    extern __shared__ __align__(128) char smem[];
+    if (!smem_layout_ok(smem)) return;  // uniform over the CTA; refused at init
+    next_may_start();
+    if (DIR == 0) fill_enc(smem);
+    else fill_dec<TWEAK>(smem);
+    wait_for_previous();
+    __syncthreads();
+    uint4* tweaks = reinterpret_cast<uint4*>(smem + (DIR == 0 ? kSmemEnc : kSmemDec));
+    bulk_chunks<NR, DIR, TWEAK, kBulkThreads / 32>(p, tweaks, cta_first(p), cta_own(p));
+}
+
+// ---------------------------------------------------------------------------
+// Large XTS and ECB encryption on two pipes at once.  The lookups keep the
+// shared-memory path 97% busy and leave two thirds of the ALU pipe and a third
+// of the issue slots idle, so four warps of every CTA encipher part of its run
+// without lookups, bitsliced: 32 blocks per lane as 128 bit-planes (see
+// bitslice_device.cuh).  Their round keys are masks in the parameter bank and
+// their spills are outside the rounds, so that they stay off the shared-memory
+// path; a warp beside its SM quarter's four table warps takes about 140 us for
+// a span of 1,024 blocks with AES-256, 43 with the quarter to itself.  The 16
+// table warps (as fast as 32 here) take the rest of the run as bulk_kernel
+// does.  The split is fixed by the launch (mix_spans): the spans come from the
+// start of the run, where all blocks exist.
+//
+// The rounds of both parts are as they measured best.  Table rounds as a loop,
+// to leave the instruction cache to the planes, wait for their keys (1 GiB of
+// AES-256: 1,660 us with a tenth on planes, 1,496 unrolled); with 8 or 12 table
+// warps of two blocks a lane the planes go faster, but the tables lose more
+// (1,637 / 1,508 us); plane masks in shared memory cost 11 us of 1,489.
+// Tables alone / mixed: AES-256-XTS of 1 GiB 1,584 / 1,474 us, 300 MiB 471 / 439,
+// 112 MiB 181 / 172; AES-128-XTS of 1 GiB 1,155 / 1,098; ECB of 1 GiB 1,573 /
+// 1,427 and 1,146 / 1,046.
+// ---------------------------------------------------------------------------
+
+// Blocks [b0, b0 + 1024), bitsliced; lane l holds blocks l, l + 32, ... .  tw:
+// 32 words of shared memory for the E_K2 of the span's data units, which has
+// at most 32 as a unit is at least 32 blocks and b0 a multiple of 32.
+template <int NR, bool TWEAK>
+__device__ __forceinline__ void bitsliced_span(const MixParams& mp, uint4* tw, uint64_t b0) {
+    const BulkParams& p = mp.b;
+    const uint32_t lane = lane_id();
+    const uint32_t bps = p.bps;
+    uint32_t u0 = 0, j0 = 0;
+    uint4 t0 = make_uint4(0, 0, 0, 0);
+    if constexpr (TWEAK) {
+        const uint64_t unit0 = div_small(b0, bps);
+        const uint32_t q = (uint32_t)(b0 - unit0 * bps) + lane;
+        const uint64_t unit = p.first_sector + unit0 + lane;
+        uint4 z = make_uint4((uint32_t)unit, (uint32_t)(unit >> 32), 0, 0);
+        const Rep4 T{lane * 4u, lane * 4u + 128u};
+        encrypt_block<NR>(z.x, z.y, z.z, z.w, T, ParamKey{p.tk});
+        __syncwarp();  // the last span's have been read
+        tw[lane] = z;
+        __syncwarp();
+        u0 = q / bps;
+        j0 = q - u0 * bps;
+        t0 = tw[u0];
+        gf128_mul_xpow(t0.x, t0.y, t0.z, t0.w, j0);
+    }
+    uint32_t S[128];
+    const uint4* in = p.src + b0 + lane;
+#pragma unroll
+    for (int i = 0; i < 32; i++) {
+        const uint4 v = in[32 * i];
+        S[i] = v.x;
+        S[32 + i] = v.y;
+        S[64 + i] = v.z;
+        S[96 + i] = v.w;
+    }
+    auto whiten = [&]() {
+        uint32_t u = u0, j = j0;
+        uint4 t = t0;
+#pragma unroll
+        for (int i = 0; i < 32; i++) {
+            S[i] ^= t.x;
+            S[32 + i] ^= t.y;
+            S[64 + i] ^= t.z;
+            S[96 + i] ^= t.w;
+            if (i == 31) break;
+            j += 32;
+            if (j >= bps) {
+                j -= bps;
+                t = tw[++u];
+                gf128_mul_xk(t.x, t.y, t.z, t.w, j);
+            } else {
+                gf128_mul_x32(t.x, t.y, t.z, t.w);
+            }
+        }
+    };
+    if constexpr (TWEAK) whiten();
+#pragma unroll
+    for (int q = 0; q < 4; q++) transpose32(S + 32 * q);
+    bs_encrypt<NR, false>(S, mp.masks);
+#pragma unroll
+    for (int q = 0; q < 4; q++) transpose32(S + 32 * q);
+    if constexpr (TWEAK) whiten();
+    uint4* out = p.dst + b0 + lane;
+#pragma unroll
+    for (int i = 0; i < 32; i++) out[32 * i] = make_uint4(S[i], S[32 + i], S[64 + i], S[96 + i]);
+}
+
+template <int NR, bool TWEAK>
+__global__ void __launch_bounds__(kMixThreads, 1) mixed_kernel(const __grid_constant__ MixParams mp) {
+    extern __shared__ __align__(128) char smem[];
+    if (!smem_layout_ok(smem)) return;
+    next_may_start();
+    fill_enc(smem);
+    wait_for_previous();
+    __syncthreads();
+    uint4* tweaks = reinterpret_cast<uint4*>(smem + kSmemEnc);
+    const uint64_t first = cta_first(mp.b);
+    const uint32_t spans = mp.spans * kMixPlaneWarps;
+    const uint32_t warp = threadIdx.x >> 5;
+    if (warp < kMixTableWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMixTableRegs));
+        bulk_chunks<NR, 0, TWEAK, kMixTableWarps>(mp.b, tweaks, first + kMixSpanChunks * spans,
+                                                  cta_own(mp.b) - kMixSpanChunks * spans);
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMixPlaneRegs));
+#pragma unroll 1
+        for (uint32_t s = warp - kMixTableWarps; s < spans; s += kMixPlaneWarps)
+            bitsliced_span<NR, TWEAK>(mp, tweaks + warp * 32u, (first + (uint64_t)kMixSpanChunks * s) << 5);
     }
 }
 
@@ -927,6 +1054,15 @@ size_t bulk_smem(int dir, bool tweak) {
     return (dir == 0 ? kSmemEnc : kSmemDec) + (tweak ? kBulkThreads * 16 : 0);
 }
 
+KernelFn<MixParams> mixed_fn(int nr, bool tweak) {
+    switch (nr) {
+        case 10: return tweak ? mixed_kernel<10, true> : mixed_kernel<10, false>;
+        case 12: return tweak ? nullptr : mixed_kernel<12, false>;  // there is no XTS-AES-192
+        case 14: return tweak ? mixed_kernel<14, true> : mixed_kernel<14, false>;
+        default: return nullptr;
+    }
+}
+
 size_t cts_smem(int dir) { return (dir == 0 ? kSmemEnc : kSmemDec) + kCtsThreads * 32; }
 
 KernelFn<CtsParams> cts_fn(int nr, int dir) {
@@ -1022,6 +1158,17 @@ cudaError_t configure_kernels() {
                 if (e != cudaSuccess) return e;
             }
         }
+        for (bool tw : {false, true}) {
+            auto fn = mixed_fn(nr, tw);
+            if (!fn) continue;
+            cudaFuncAttributes attr;
+            cudaError_t e = cudaFuncGetAttributes(&attr, fn);
+            if (e != cudaSuccess) return e;
+            // what the register shares of its warps are drawn from
+            if (attr.numRegs != kMixLaunchRegs) return cudaErrorInvalidConfiguration;
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMix);
+            if (e != cudaSuccess) return e;
+        }
         cudaError_t e = cudaFuncSetAttribute(cbc_fn(nr, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemEnc);
         if (e != cudaSuccess) return e;
@@ -1053,6 +1200,21 @@ cudaError_t upload_tables(const uint32_t* te0, const uint32_t* td0, const uint32
     return e;
 }
 
+// Spans that each bitsliced warp of a CTA takes from a run of cta_chunks
+// 32-block chunks; 0: the call stays on the tables.  A warp that takes one span
+// too many costs the call up to a span's time, so a span is given for every
+// so many chunks as the table warps encipher meanwhile, rounded down.  1 GiB
+// (13,797 chunks a CTA) of AES-256-XTS by spans per warp: 0 1,584 us, 10 1,475,
+// 11 1,527; of AES-128 0 1,155, 9 1,099, 10 1,160; of ECB, which forms no
+// tweaks, with AES-256 0 1,573, 10 1,443, 11 1,428, with AES-128 9 1,066, 11
+// 1,046.  Units under 512 bytes have more tweaks than a span has lanes, and
+// pages that cross the host link are bound by it.
+uint32_t mix_spans(uint32_t cta_chunks, int nr, int dir, bool tweak, uint32_t bps, bool link) {
+    if (dir != 0 || link || (tweak && bps < 32)) return 0;
+    const uint32_t per_span = tweak ? (nr == 14 ? 1300 : 1400) : (nr == 14 ? 1200 : 1250);
+    return cta_chunks / per_span;
+}
+
 static cudaError_t launch_bulk(const BulkParams& params, int nr, int dir, bool tweak, int num_sms, cudaStream_t s) {
     auto fn = bulk_fn(nr, dir, tweak);
     if (!fn) return cudaErrorInvalidValue;
@@ -1062,6 +1224,13 @@ static cudaError_t launch_bulk(const BulkParams& params, int nr, int dir, bool t
     if (chunks / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     p.cta_chunks = (uint32_t)(chunks / grid);
     p.cta_rest = (uint32_t)(chunks % grid);
+    if (const uint32_t spans = mix_spans(p.cta_chunks, nr, dir, tweak, p.bps, p.link != 0)) {
+        MixParams mp;
+        mp.b = p;
+        mp.spans = spans;
+        for (int i = 0; i < 128 * (nr + 1); i++) mp.masks[i] = (p.rk[i >> 5] >> (i & 31)) & 1u ? ~0u : 0u;
+        return launch<MixParams>(mixed_fn(nr, tweak), grid, kMixThreads, kSmemMix, s, mp);
+    }
     return launch(fn, grid, kBulkThreads, bulk_smem(dir, tweak), s, p);
 }
 

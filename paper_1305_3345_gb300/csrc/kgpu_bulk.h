@@ -1,7 +1,8 @@
 // Parameter blocks and launch entry points of the bulk kernels (kgpu_bulk.cu):
 // one kernel per mode, direction and key size, for the per-call transforms.
 // Kept apart from the batched and serving formats so that the bulk kernels'
-// sources are exactly aes_device.cuh, kgpu_bulk.cu and this header.
+// sources are exactly aes_device.cuh, bitslice_device.cuh, sbox_circuit.cuh,
+// kgpu_bulk.cu and this header.
 #pragma once
 #include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
@@ -20,6 +21,21 @@ constexpr size_t kSmemDec = 3 * kRegionBytes;  // regions A, B, C
 
 // Threads per CTA of the bulk kernels (one CTA per SM).
 constexpr int kBulkThreads = 1024;
+
+// Large XTS / ECB encryptions on tables and bit-planes at once (mixed_kernel):
+// 16 warps make table lookups and 4 run the bitsliced cipher.  The CTA is
+// launched with 96 registers a thread, which setmaxnreg hands out again as 64
+// and 224; the shares may not exceed what the launch has, or the warps that
+// ask for more would wait for ever.
+constexpr int kMixTableWarps = 16, kMixPlaneWarps = 4;
+constexpr int kMixThreads = (kMixTableWarps + kMixPlaneWarps) * 32;
+constexpr int kMixLaunchRegs = 96, kMixTableRegs = 64, kMixPlaneRegs = 224;
+static_assert(kMixTableWarps * kMixTableRegs + kMixPlaneWarps * kMixPlaneRegs <=
+                  (kMixTableWarps + kMixPlaneWarps) * kMixLaunchRegs,
+              "register shares exceed the launch's registers");
+static_assert(kMixTableWarps % 4 == 0 && kMixPlaneWarps % 4 == 0, "setmaxnreg acts on whole warpgroups");
+constexpr uint32_t kMixSpanChunks = 32;  // a bitsliced span in 32-block chunks
+constexpr size_t kSmemMix = kSmemEnc + (kMixTableWarps + kMixPlaneWarps) * 512;  // E_K2 of 32 units per warp
 
 // CBC encryption with a chain split over 2 or 4 lanes: at most 16 warps per CTA.
 constexpr int kCbcSplitThreads = 512;
@@ -64,10 +80,19 @@ struct BulkParams {
     uint32_t bps;           // blocks per data unit (XTS)
     uint32_t cta_rest;      // set by the launch: CTA b has cta_chunks 32-block chunks,
     uint32_t cta_chunks;    // one more if b < cta_rest
-    uint32_t pad0;
+    uint32_t link;          // 1: pages cross the host link, which bounds the call
     uint64_t first_sector;  // number of the first data unit (XTS)
     uint32_t rk[kMaxRoundKeyWords];  // data key schedule (encryption or decryption order)
     uint32_t tk[kMaxRoundKeyWords];  // tweak key schedule (always encryption)
+};
+
+// Parameters of the mixed kernel: the same, the spans that each bitsliced warp
+// takes from the start of its CTA's run, and the data key's plane masks (bit i
+// of round key r as 0 or ~0 at 128 r + i).
+struct MixParams {
+    BulkParams b;
+    uint32_t spans;
+    alignas(16) uint32_t masks[15 * 128];
 };
 
 // Parameters of the CBC kernels.

@@ -179,6 +179,7 @@ cudaError_t launch_one(const kgpu_ctx* ctx, const ReqDesc& d, const HostKey& k, 
     if (d.mode == KGPU_MODE_XTS || d.mode == KGPU_MODE_ECB) {
         BulkParams p;
         fill_bulk(&p, k, (int)d.dir, d.src, d.dst, d.nblocks * 16, (size_t)d.unit_blocks * 16, d.first_sector);
+        p.link = (d.flags & (kDescSrcHost | kDescDstHost)) != 0;
         return d.mode == KGPU_MODE_XTS ? launch_xts(p, k.nr, (int)d.dir, ctx->num_sms, s)
                                        : launch_ecb(p, k.nr, (int)d.dir, ctx->num_sms, s);
     }

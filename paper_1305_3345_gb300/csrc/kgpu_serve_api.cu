@@ -1006,6 +1006,7 @@ int kgpu_replay_launches(kgpu_ctx* ctx, const kgpu_request* reqs, const uint64_t
             const HostKey& k = keys[d.key];
             BulkParams p;
             fill_bulk(&p, k, (int)d.dir, d.src, d.dst, d.nblocks * 16, (size_t)d.unit_blocks * 16, d.first_sector);
+            p.link = (d.flags & (kDescSrcHost | kDescDstHost)) != 0;
             e = d.mode == KGPU_MODE_XTS ? launch_xts(p, k.nr, (int)d.dir, ctx->num_sms, s)
                                         : launch_ecb(p, k.nr, (int)d.dir, ctx->num_sms, s);
         } else {
