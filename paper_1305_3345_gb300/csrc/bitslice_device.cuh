@@ -59,6 +59,31 @@ __device__ __noinline__ static Byte8 sbox_call(Byte8 b) {
     return b;
 }
 
+// The inverse of the S-box's affine map (FIPS-197 section 5.3.2): bit i of the
+// result is x_(i+2) ^ x_(i+5) ^ x_(i+7), inverted for i = 0 and 2.
+__device__ __forceinline__ void inverse_affine(uint32_t* x) {
+    uint32_t y[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) y[i] = x[(i + 2) & 7] ^ x[(i + 5) & 7] ^ x[(i + 7) & 7];
+    y[0] = ~y[0];
+    y[2] = ~y[2];
+#pragma unroll
+    for (int i = 0; i < 8; i++) x[i] = y[i];
+}
+
+// InvSubBytes from the same circuit: with S = A o I, A the affine map and I
+// the field inversion, which is its own inverse, S^-1 = I o A^-1 =
+// A^-1 o S o A^-1.  Sixteen three-input XORs a byte more than SubBytes.
+__device__ __forceinline__ void inv_sub_bytes(uint32_t (&S)[128]) {
+#pragma unroll
+    for (int p = 0; p < 16; p++) {
+        uint32_t* x = S + 8 * p;
+        inverse_affine(x);
+        sbox_circuit(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+        inverse_affine(x);
+    }
+}
+
 template <bool CALL>
 __device__ __forceinline__ void sub_bytes(uint32_t (&S)[128]) {
 #pragma unroll
@@ -129,6 +154,70 @@ __device__ __forceinline__ void shift_mix_key(uint32_t (&S)[128], const uint32_t
     for (int i = 0; i < 128; i++) S[i] = N[i];
 }
 
+// u times x on planes.
+__device__ __forceinline__ void xtime_planes(const uint32_t* u, uint32_t* y) {
+    y[0] = u[7];
+    y[1] = u[0] ^ u[7];
+    y[2] = u[1];
+    y[3] = u[2] ^ u[7];
+    y[4] = u[3] ^ u[7];
+    y[5] = u[4];
+    y[6] = u[5];
+    y[7] = u[6];
+}
+
+// InvShiftRows, then InvMixColumns (when MIX) and AddRoundKey: the order of the
+// equivalent inverse cipher.  InvMixColumns is MixColumns after
+// a_r ^= x^2 (a_r ^ a_{r+2}).
+template <bool MIX>
+__device__ __forceinline__ void inv_shift_mix_key(uint32_t (&S)[128], const uint32_t* k) {
+    uint32_t N[128];
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        uint32_t a[4][8];
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+            for (int b = 0; b < 8; b++) a[r][b] = S[8 * (r + 4 * ((c - r) & 3)) + b];
+        if constexpr (MIX) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                uint32_t v[8], x1[8], x2[8];
+#pragma unroll
+                for (int b = 0; b < 8; b++) v[b] = a[h][b] ^ a[h + 2][b];
+                xtime_planes(v, x1);
+                xtime_planes(x1, x2);
+#pragma unroll
+                for (int b = 0; b < 8; b++) {
+                    a[h][b] ^= x2[b];
+                    a[h + 2][b] ^= x2[b];
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            uint32_t x2[8];
+            if constexpr (MIX) {
+                uint32_t u[8];
+#pragma unroll
+                for (int b = 0; b < 8; b++) u[b] = a[r][b] ^ a[(r + 1) & 3][b];
+                xtime_planes(u, x2);
+            }
+#pragma unroll
+            for (int b = 0; b < 8; b++) {
+                const uint32_t kb = k[8 * (r + 4 * c) + b];
+                if constexpr (MIX)
+                    N[8 * (r + 4 * c) + b] =
+                        x2[b] ^ a[(r + 1) & 3][b] ^ (a[(r + 2) & 3][b] ^ a[(r + 3) & 3][b]) ^ kb;
+                else
+                    N[8 * (r + 4 * c) + b] = a[r][b] ^ kb;
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 128; i++) S[i] = N[i];
+}
+
 // The forward cipher on planes; km holds (NR + 1) x 128 round-key masks, in
 // shared memory or in the parameter bank.  CALL: the S-box as a function.  The round loop is not unrolled: one round is ~2,000
 // instructions, and 14 unrolled rounds would not fit the instruction cache.
@@ -146,6 +235,22 @@ __device__ __forceinline__ void bs_encrypt(uint32_t (&S)[128], const uint32_t* k
             shift_mix_key<true>(S, km + 128 * r);
         else
             shift_mix_key<false>(S, km + 128 * r);
+    }
+}
+
+// The equivalent inverse cipher (FIPS-197 section 5.3.5) on planes; km holds the
+// masks of its schedule.
+template <int NR>
+__device__ __forceinline__ void bs_decrypt(uint32_t (&S)[128], const uint32_t* km) {
+#pragma unroll
+    for (int i = 0; i < 128; i++) S[i] ^= km[i];
+#pragma unroll 1
+    for (int r = 1; r <= NR; r++) {
+        inv_sub_bytes(S);
+        if (r < NR)
+            inv_shift_mix_key<true>(S, km + 128 * r);
+        else
+            inv_shift_mix_key<false>(S, km + 128 * r);
     }
 }
 

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_cons
 }
 
 // ---------------------------------------------------------------------------
-// Large XTS and ECB encryption on two pipes at once.  The lookups keep the
+// Large XTS and ECB calls on two pipes at once.  The lookups keep the
 // shared-memory path 97% busy and leave two thirds of the ALU pipe and a third
 // of the issue slots idle, so four warps of every CTA encipher part of its run
 // without lookups, bitsliced: 32 blocks per lane as 128 bit-planes (see
@@ -250,13 +250,36 @@ __global__ void __launch_bounds__(kBulkThreads, 1) bulk_kernel(const __grid_cons
 // (1,637 / 1,508 us); plane masks in shared memory cost 11 us of 1,489.
 // Tables alone / mixed: AES-256-XTS of 1 GiB 1,584 / 1,474 us, 300 MiB 471 / 439,
 // 112 MiB 181 / 172; AES-128-XTS of 1 GiB 1,155 / 1,098; ECB of 1 GiB 1,573 /
-// 1,427 and 1,146 / 1,046.
+// 1,427 and 1,146 / 1,046.  Decryption, whose inverse S-box and InvMixColumns are
+// a fifth more work on the planes: AES-256-XTS of 1 GiB 1,591 / 1,524, 130 MiB
+// 208 / 201; AES-128-XTS 1,165 / 1,130; ECB 1,582 / 1,471 and 1,156 / 1,071.
 // ---------------------------------------------------------------------------
+
+__device__ __forceinline__ void load_span(uint32_t (&S)[128], const uint4* in) {
+#pragma unroll
+    for (int i = 0; i < 32; i++) {
+        const uint4 v = in[32 * i];
+        S[i] = v.x;
+        S[32 + i] = v.y;
+        S[64 + i] = v.z;
+        S[96 + i] = v.w;
+    }
+}
+
+template <int NR, int DIR>
+__device__ __forceinline__ void cipher_span(uint32_t (&S)[128], const uint32_t* masks) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) transpose32(S + 32 * q);
+    if constexpr (DIR == 0) bs_encrypt<NR, false>(S, masks);
+    else bs_decrypt<NR>(S, masks);
+#pragma unroll
+    for (int q = 0; q < 4; q++) transpose32(S + 32 * q);
+}
 
 // Blocks [b0, b0 + 1024), bitsliced; lane l holds blocks l, l + 32, ... .  tw:
 // 32 words of shared memory for the E_K2 of the span's data units, which has
 // at most 32 as a unit is at least 32 blocks and b0 a multiple of 32.
-template <int NR, bool TWEAK>
+template <int NR, int DIR, bool TWEAK>
 __device__ __forceinline__ void bitsliced_span(const MixParams& mp, uint4* tw, uint64_t b0) {
     const BulkParams& p = mp.b;
     const uint32_t lane = lane_id();
@@ -268,8 +291,10 @@ __device__ __forceinline__ void bitsliced_span(const MixParams& mp, uint4* tw, u
         const uint32_t q = (uint32_t)(b0 - unit0 * bps) + lane;
         const uint64_t unit = p.first_sector + unit0 + lane;
         uint4 z = make_uint4((uint32_t)unit, (uint32_t)(unit >> 32), 0, 0);
-        const Rep4 T{lane * 4u, lane * 4u + 128u};
-        encrypt_block<NR>(z.x, z.y, z.z, z.w, T, ParamKey{p.tk});
+        if constexpr (DIR == 0)
+            encrypt_block<NR>(z.x, z.y, z.z, z.w, Rep4{lane * 4u, lane * 4u + 128u}, ParamKey{p.tk});
+        else
+            encrypt_block<NR>(z.x, z.y, z.z, z.w, Rep1<2>{lane * 4u + 128u}, ParamKey{p.tk});
         __syncwarp();  // the last span's have been read
         tw[lane] = z;
         __syncwarp();
@@ -279,15 +304,7 @@ __device__ __forceinline__ void bitsliced_span(const MixParams& mp, uint4* tw, u
         gf128_mul_xpow(t0.x, t0.y, t0.z, t0.w, j0);
     }
     uint32_t S[128];
-    const uint4* in = p.src + b0 + lane;
-#pragma unroll
-    for (int i = 0; i < 32; i++) {
-        const uint4 v = in[32 * i];
-        S[i] = v.x;
-        S[32 + i] = v.y;
-        S[64 + i] = v.z;
-        S[96 + i] = v.w;
-    }
+    load_span(S, p.src + b0 + lane);
     auto whiten = [&]() {
         uint32_t u = u0, j = j0;
         uint4 t = t0;
@@ -309,38 +326,35 @@ __device__ __forceinline__ void bitsliced_span(const MixParams& mp, uint4* tw, u
         }
     };
     if constexpr (TWEAK) whiten();
-#pragma unroll
-    for (int q = 0; q < 4; q++) transpose32(S + 32 * q);
-    bs_encrypt<NR, false>(S, mp.masks);
-#pragma unroll
-    for (int q = 0; q < 4; q++) transpose32(S + 32 * q);
+    cipher_span<NR, DIR>(S, mp.masks);
     if constexpr (TWEAK) whiten();
     uint4* out = p.dst + b0 + lane;
 #pragma unroll
     for (int i = 0; i < 32; i++) out[32 * i] = make_uint4(S[i], S[32 + i], S[64 + i], S[96 + i]);
 }
 
-template <int NR, bool TWEAK>
+template <int NR, int DIR, bool TWEAK>
 __global__ void __launch_bounds__(kMixThreads, 1) mixed_kernel(const __grid_constant__ MixParams mp) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
     next_may_start();
-    fill_enc(smem);
+    if (DIR == 0) fill_enc(smem);
+    else fill_dec<TWEAK>(smem);
     wait_for_previous();
     __syncthreads();
-    uint4* tweaks = reinterpret_cast<uint4*>(smem + kSmemEnc);
+    uint4* tweaks = reinterpret_cast<uint4*>(smem + (DIR == 0 ? kSmemEnc : kSmemDec));
     const uint64_t first = cta_first(mp.b);
     const uint32_t spans = mp.spans * kMixPlaneWarps;
     const uint32_t warp = threadIdx.x >> 5;
     if (warp < kMixTableWarps) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMixTableRegs));
-        bulk_chunks<NR, 0, TWEAK, kMixTableWarps>(mp.b, tweaks, first + kMixSpanChunks * spans,
-                                                  cta_own(mp.b) - kMixSpanChunks * spans);
+        bulk_chunks<NR, DIR, TWEAK, kMixTableWarps>(mp.b, tweaks, first + kMixSpanChunks * spans,
+                                                    cta_own(mp.b) - kMixSpanChunks * spans);
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMixPlaneRegs));
 #pragma unroll 1
         for (uint32_t s = warp - kMixTableWarps; s < spans; s += kMixPlaneWarps)
-            bitsliced_span<NR, TWEAK>(mp, tweaks + warp * 32u, (first + (uint64_t)kMixSpanChunks * s) << 5);
+            bitsliced_span<NR, DIR, TWEAK>(mp, tweaks + warp * 32u, (first + (uint64_t)kMixSpanChunks * s) << 5);
     }
 }
 
@@ -359,28 +373,16 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_kernel(const __grid_cons
 // touch, and every warp reads that block before the barrier that precedes the
 // first store.
 // ---------------------------------------------------------------------------
-template <int NR>
-__global__ void __launch_bounds__(kBulkThreads, 1) cbc_dec_kernel(const __grid_constant__ CbcParams p) {
-    extern __shared__ __align__(128) char smem[];
-    if (!smem_layout_ok(smem)) return;
-    next_may_start();
-    fill_dec<false>(smem);
-    wait_for_previous();
-
+template <int NR, int WARPS>
+__device__ __forceinline__ void cbc_dec_chunks(const CbcParams& p, uint64_t b0, uint64_t bend) {
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
-    constexpr uint32_t kWarps = kBulkThreads / 32;
+    constexpr uint32_t kWarps = WARPS;
     const Rep4 T{lane * 4u, lane * 4u + 128u};
     const Rep1<2> IS{lane * 4u};
     const ParamKey K{p.rk};
 
-    // this CTA's blocks [b0, bend): pages in place, else 32-block chunks
     const uint32_t bpp = p.bpp;
-    const uint64_t item = p.src == p.dst ? bpp : 32u;
-    const uint64_t first = (uint64_t)p.cta_items * blockIdx.x + min(blockIdx.x, p.cta_rest);
-    const uint32_t own = p.cta_items + (blockIdx.x < p.cta_rest ? 1u : 0u);
-    const uint64_t b0 = first * item;
-    const uint64_t bend = min(b0 + own * item, p.npages * bpp);
     const uint32_t chunks = (uint32_t)((bend - b0 + 31) >> 5);
     const uint32_t a = (uint32_t)((uint64_t)chunks * warp / kWarps);
     const uint32_t e = (uint32_t)((uint64_t)chunks * (warp + 1) / kWarps);
@@ -390,7 +392,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) cbc_dec_kernel(const __grid_c
     const bool some = a < e && blk < bend;
     uint4 carry = some && lane == 0 && j ? p.src[blk - 1] : make_uint4(0, 0, 0, 0);
     uint4 nxt = some ? p.src[blk] : make_uint4(0, 0, 0, 0);
-    __syncthreads();  // the tables are filled and every carry is read
+    if (WARPS * 32 == kBulkThreads) __syncthreads();  // the tables are filled and every carry is read
 
     for (uint32_t i = a; i < e; ++i) {
         const bool valid = blk < bend;
@@ -421,6 +423,74 @@ __global__ void __launch_bounds__(kBulkThreads, 1) cbc_dec_kernel(const __grid_c
             uint32_t ns = j / bpp;
             page += ns;
             j -= ns * bpp;
+        }
+    }
+}
+
+// This CTA's blocks [b0, bend): pages in place, else 32-block chunks.
+__device__ __forceinline__ void cta_blocks(const CbcParams& p, uint64_t& b0, uint64_t& bend) {
+    const uint64_t item = p.src == p.dst ? p.bpp : 32u;
+    const uint64_t first = (uint64_t)p.cta_items * blockIdx.x + min(blockIdx.x, p.cta_rest);
+    const uint32_t own = p.cta_items + (blockIdx.x < p.cta_rest ? 1u : 0u);
+    b0 = first * item;
+    bend = min(b0 + own * item, p.npages * p.bpp);
+}
+
+template <int NR>
+__global__ void __launch_bounds__(kBulkThreads, 1) cbc_dec_kernel(const __grid_constant__ CbcParams p) {
+    extern __shared__ __align__(128) char smem[];
+    if (!smem_layout_ok(smem)) return;
+    next_may_start();
+    fill_dec<false>(smem);
+    wait_for_previous();
+    uint64_t b0, bend;
+    cta_blocks(p, b0, bend);
+    cbc_dec_chunks<NR, kBulkThreads / 32>(p, b0, bend);
+}
+
+// Large CBC decryption out of place on tables and bit-planes, as mixed_kernel.
+// A span's lanes read the block before each of theirs again once they have
+// deciphered it; pages are of at least 32 blocks, so that a lane enters at most
+// one from one block to its next.  4-KiB pages, tables alone / mixed: AES-128 of
+// 1 GiB 1,189 / 1,121 us, of 130 MiB 156 / 150; AES-256 1,616 / 1,541.
+template <int NR>
+__global__ void __launch_bounds__(kMixThreads, 1) mixed_cbc_dec_kernel(const __grid_constant__ MixCbcParams mp) {
+    extern __shared__ __align__(128) char smem[];
+    if (!smem_layout_ok(smem)) return;
+    next_may_start();
+    fill_dec<false>(smem);
+    wait_for_previous();
+    __syncthreads();
+    const CbcParams& p = mp.c;
+    uint64_t b0, bend;
+    cta_blocks(p, b0, bend);
+    const uint32_t spans = mp.spans * kMixPlaneWarps;
+    const uint32_t warp = threadIdx.x >> 5;
+    if (warp < kMixTableWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMixTableRegs));
+        cbc_dec_chunks<NR, kMixTableWarps>(p, b0 + (uint64_t)kBsSpan * spans, bend);
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMixPlaneRegs));
+        const uint32_t bpp = p.bpp;
+#pragma unroll 1
+        for (uint32_t s = warp - kMixTableWarps; s < spans; s += kMixPlaneWarps) {
+            const uint64_t n = b0 + (uint64_t)kBsSpan * s + lane_id();
+            uint32_t S[128];
+            load_span(S, p.src + n);
+            cipher_span<NR, 1>(S, mp.masks);
+            uint64_t page = div_small(n, bpp);
+            uint32_t j = (uint32_t)(n - page * bpp);
+#pragma unroll
+            for (int i = 0; i < 32; i++) {
+                const uint4 prev = j ? p.src[n + 32 * i - 1] : p.ivs[page];
+                p.dst[n + 32 * i] =
+                    make_uint4(S[i] ^ prev.x, S[32 + i] ^ prev.y, S[64 + i] ^ prev.z, S[96 + i] ^ prev.w);
+                j += 32;
+                if (j >= bpp) {
+                    j -= bpp;
+                    page++;
+                }
+            }
         }
     }
 }
@@ -1054,13 +1124,47 @@ size_t bulk_smem(int dir, bool tweak) {
     return (dir == 0 ? kSmemEnc : kSmemDec) + (tweak ? kBulkThreads * 16 : 0);
 }
 
-KernelFn<MixParams> mixed_fn(int nr, bool tweak) {
+template <int NR>
+KernelFn<MixParams> pick_mixed(int dir, bool tweak) {
+    if (tweak) return dir == 0 ? mixed_kernel<NR, 0, true> : mixed_kernel<NR, 1, true>;
+    return dir == 0 ? mixed_kernel<NR, 0, false> : mixed_kernel<NR, 1, false>;
+}
+
+KernelFn<MixParams> mixed_fn(int nr, int dir, bool tweak) {
     switch (nr) {
-        case 10: return tweak ? mixed_kernel<10, true> : mixed_kernel<10, false>;
-        case 12: return tweak ? nullptr : mixed_kernel<12, false>;  // there is no XTS-AES-192
-        case 14: return tweak ? mixed_kernel<14, true> : mixed_kernel<14, false>;
+        case 10: return pick_mixed<10>(dir, tweak);
+        case 12:  // there is no XTS-AES-192
+            if (tweak) return nullptr;
+            return dir == 0 ? mixed_kernel<12, 0, false> : mixed_kernel<12, 1, false>;
+        case 14: return pick_mixed<14>(dir, tweak);
         default: return nullptr;
     }
+}
+
+KernelFn<MixCbcParams> mixed_cbc_dec_fn(int nr) {
+    switch (nr) {
+        case 10: return mixed_cbc_dec_kernel<10>;
+        case 12: return mixed_cbc_dec_kernel<12>;
+        case 14: return mixed_cbc_dec_kernel<14>;
+        default: return nullptr;
+    }
+}
+
+size_t mixed_smem(int dir) { return (dir == 0 ? kSmemEnc : kSmemDec) + kMixTweakBytes; }
+
+template <class P>
+cudaError_t configure_mixed(KernelFn<P> fn, size_t smem) {
+    if (!fn) return cudaSuccess;
+    cudaFuncAttributes attr;
+    cudaError_t e = cudaFuncGetAttributes(&attr, fn);
+    if (e != cudaSuccess) return e;
+    // what the register shares of its warps are drawn from
+    if (attr.numRegs != kMixLaunchRegs) return cudaErrorInvalidConfiguration;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
+void plane_masks(uint32_t* masks, const uint32_t* rk, int nr) {
+    for (int i = 0; i < 128 * (nr + 1); i++) masks[i] = (rk[i >> 5] >> (i & 31)) & 1u ? ~0u : 0u;
 }
 
 size_t cts_smem(int dir) { return (dir == 0 ? kSmemEnc : kSmemDec) + kCtsThreads * 32; }
@@ -1156,20 +1260,13 @@ cudaError_t configure_kernels() {
                 cudaError_t e = cudaFuncSetAttribute(bulk_fn(nr, dir, tw), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)bulk_smem(dir, tw));
                 if (e != cudaSuccess) return e;
+                e = configure_mixed(mixed_fn(nr, dir, tw), mixed_smem(dir));
+                if (e != cudaSuccess) return e;
             }
         }
-        for (bool tw : {false, true}) {
-            auto fn = mixed_fn(nr, tw);
-            if (!fn) continue;
-            cudaFuncAttributes attr;
-            cudaError_t e = cudaFuncGetAttributes(&attr, fn);
-            if (e != cudaSuccess) return e;
-            // what the register shares of its warps are drawn from
-            if (attr.numRegs != kMixLaunchRegs) return cudaErrorInvalidConfiguration;
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMix);
-            if (e != cudaSuccess) return e;
-        }
-        cudaError_t e = cudaFuncSetAttribute(cbc_fn(nr, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = configure_mixed(mixed_cbc_dec_fn(nr), kSmemDec);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(cbc_fn(nr, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemEnc);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(cbc_fn(nr, false), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDec);
@@ -1207,11 +1304,16 @@ cudaError_t upload_tables(const uint32_t* te0, const uint32_t* td0, const uint32
 // (13,797 chunks a CTA) of AES-256-XTS by spans per warp: 0 1,584 us, 10 1,475,
 // 11 1,527; of AES-128 0 1,155, 9 1,099, 10 1,160; of ECB, which forms no
 // tweaks, with AES-256 0 1,573, 10 1,443, 11 1,428, with AES-128 9 1,066, 11
-// 1,046.  Units under 512 bytes have more tweaks than a span has lanes, and
+// 1,046; of decryption with AES-256-XTS 0 1,591, 8 1,524, 9 1,540, with AES-128
+// 0 1,165, 7 1,130, 8 1,135; of CBC decryption with AES-256 0 1,616, 10 1,541, 11
+// 1,563, with AES-128 0 1,189, 10 1,121, 11 1,165.  Units under 512 bytes have more tweaks than a span has lanes, and
 // pages that cross the host link are bound by it.
-uint32_t mix_spans(uint32_t cta_chunks, int nr, int dir, bool tweak, uint32_t bps, bool link) {
-    if (dir != 0 || link || (tweak && bps < 32)) return 0;
-    const uint32_t per_span = tweak ? (nr == 14 ? 1300 : 1400) : (nr == 14 ? 1200 : 1250);
+uint32_t mix_spans(uint32_t cta_chunks, int nr, int dir, bool tweak, uint32_t unit_blocks, bool link) {
+    if (link || unit_blocks < 32 || (tweak && nr == 12)) return 0;
+    const bool big = nr == 14;
+    uint32_t per_span;
+    if (dir == 0) per_span = tweak ? (big ? 1300 : 1400) : (big ? 1200 : 1250);
+    else per_span = tweak ? (big ? 1600 : 1800) : 1300;
     return cta_chunks / per_span;
 }
 
@@ -1224,12 +1326,12 @@ static cudaError_t launch_bulk(const BulkParams& params, int nr, int dir, bool t
     if (chunks / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     p.cta_chunks = (uint32_t)(chunks / grid);
     p.cta_rest = (uint32_t)(chunks % grid);
-    if (const uint32_t spans = mix_spans(p.cta_chunks, nr, dir, tweak, p.bps, p.link != 0)) {
+    if (const uint32_t spans = mix_spans(p.cta_chunks, nr, dir, tweak, tweak ? p.bps : 32, p.link != 0)) {
         MixParams mp;
         mp.b = p;
         mp.spans = spans;
-        for (int i = 0; i < 128 * (nr + 1); i++) mp.masks[i] = (p.rk[i >> 5] >> (i & 31)) & 1u ? ~0u : 0u;
-        return launch<MixParams>(mixed_fn(nr, tweak), grid, kMixThreads, kSmemMix, s, mp);
+        plane_masks(mp.masks, p.rk, nr);
+        return launch(mixed_fn(nr, dir, tweak), grid, kMixThreads, mixed_smem(dir), s, mp);
     }
     return launch(fn, grid, kBulkThreads, bulk_smem(dir, tweak), s, p);
 }
@@ -1252,6 +1354,13 @@ cudaError_t launch_cbc_dec(const CbcParams& p, int nr, int num_sms, cudaStream_t
     if (items / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     q.cta_items = (uint32_t)(items / grid);
     q.cta_rest = (uint32_t)(items % grid);
+    if (const uint32_t spans = in_place ? 0 : mix_spans(q.cta_items, nr, 1, false, p.bpp, p.link != 0)) {
+        MixCbcParams mp;
+        mp.c = q;
+        mp.spans = spans;
+        plane_masks(mp.masks, q.rk, nr);
+        return launch(mixed_cbc_dec_fn(nr), grid, kMixThreads, kSmemDec, s, mp);
+    }
     return launch(fn, grid, kBulkThreads, kSmemDec, s, q);
 }
 

@@ -22,7 +22,7 @@ constexpr size_t kSmemDec = 3 * kRegionBytes;  // regions A, B, C
 // Threads per CTA of the bulk kernels (one CTA per SM).
 constexpr int kBulkThreads = 1024;
 
-// Large XTS / ECB encryptions on tables and bit-planes at once (mixed_kernel):
+// Large calls on tables and bit-planes at once (mixed_kernel, mixed_cbc_dec_kernel):
 // 16 warps make table lookups and 4 run the bitsliced cipher.  The CTA is
 // launched with 96 registers a thread, which setmaxnreg hands out again as 64
 // and 224; the shares may not exceed what the launch has, or the warps that
@@ -35,7 +35,7 @@ static_assert(kMixTableWarps * kMixTableRegs + kMixPlaneWarps * kMixPlaneRegs <=
               "register shares exceed the launch's registers");
 static_assert(kMixTableWarps % 4 == 0 && kMixPlaneWarps % 4 == 0, "setmaxnreg acts on whole warpgroups");
 constexpr uint32_t kMixSpanChunks = 32;  // a bitsliced span in 32-block chunks
-constexpr size_t kSmemMix = kSmemEnc + (kMixTableWarps + kMixPlaneWarps) * 512;  // E_K2 of 32 units per warp
+constexpr size_t kMixTweakBytes = (kMixTableWarps + kMixPlaneWarps) * 512;  // E_K2 of 32 units per warp
 
 // CBC encryption with a chain split over 2 or 4 lanes: at most 16 warps per CTA.
 constexpr int kCbcSplitThreads = 512;
@@ -104,7 +104,7 @@ struct CbcParams {
     uint32_t bpp;           // blocks per page
     uint32_t cta_rest;      // set by the decryption launch: CTA b has cta_items pages or
     uint32_t cta_items;     // chunks, one more if b < cta_rest
-    uint32_t pad0;
+    uint32_t link;          // 1: pages cross the host link
     uint32_t rk[kMaxRoundKeyWords];
 };
 
@@ -119,6 +119,12 @@ struct CbcTmaParams {
     uint32_t bpp;      // blocks per page, a multiple of 8
     uint32_t pad0;
     uint32_t rk[kMaxRoundKeyWords];
+};
+
+struct MixCbcParams {
+    CbcParams c;
+    uint32_t spans;
+    alignas(16) uint32_t masks[15 * 128];
 };
 
 // XTS with ciphertext stealing: data units of du bytes, du >= 16 and not a

@@ -520,7 +520,9 @@ void split_chains(ReqDesc* descs, uint32_t n, const Codes& refused, uint64_t war
 // handed out last runs alone at the end.  So every CBC-encryption request
 // runs before the tail reserve, the largest other requests holding their
 // last reserve_tiles tiles (two per resident warp: enough short work to keep
-// every warp busy while the long tiles finish).  Ties keep submission order.
+// every warp busy while the long tiles finish); plan_batch, whose kernel keeps a
+// queue for CBC encryption, asks for a reserve of everything.  Ties keep
+// submission order.
 // Allocation-free.  Returns the total tile count.
 template <class Codes>
 uint64_t order_batch(const ReqDesc* descs, uint32_t n, const Codes& codes, uint64_t reserve_tiles, uint64_t* prefix,

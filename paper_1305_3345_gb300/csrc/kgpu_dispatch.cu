@@ -190,6 +190,7 @@ cudaError_t launch_one(const kgpu_ctx* ctx, const ReqDesc& d, const HostKey& k, 
     p.ivs = d.ivs;
     p.npages = d.nblocks / d.unit_blocks;
     p.bpp = d.unit_blocks;
+    p.link = (d.flags & (kDescSrcHost | kDescDstHost)) != 0;
     const bool enc = d.mode == KGPU_MODE_CBC_ENC;
     std::memcpy(p.rk, enc ? k.enc : k.dec, sizeof(p.rk));
     return enc ? launch_cbc_enc(p, k.nr, ctx->num_sms, s) : launch_cbc_dec(p, k.nr, ctx->num_sms, s);

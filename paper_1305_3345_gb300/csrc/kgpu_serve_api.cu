@@ -1018,6 +1018,7 @@ int kgpu_replay_launches(kgpu_ctx* ctx, const kgpu_request* reqs, const uint64_t
             p.ivs = d.ivs;
             p.npages = d.nblocks / d.unit_blocks;
             p.bpp = d.unit_blocks;
+            p.link = (d.flags & (kDescSrcHost | kDescDstHost)) != 0;
             const bool enc = d.mode == KGPU_MODE_CBC_ENC;
             std::memcpy(p.rk, enc ? k.enc : k.dec, sizeof(p.rk));
             e = enc ? launch_cbc_enc(p, k.nr, ctx->num_sms, s) : launch_cbc_dec(p, k.nr, ctx->num_sms, s);
