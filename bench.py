@@ -155,6 +155,20 @@ def recorded_traffic():
     return rec.get("dram_bytes_per_launch")
 
 
+# 512-byte chunks a CTA (one per SM) needs for each span of 32 chunks that each
+# of its four bitsliced warps takes off the tables: the launch rule of the bulk
+# kernels (mix_spans in kgpu_bulk.cu)
+CHUNKS_PER_SPAN = {"aes256_xts_enc": 1300, "aes128_xts_enc": 1400, "aes256_xts_dec": 1600, "aes128_xts_dec": 1800,
+                   "aes128_ecb_enc": 1250, "aes128_cbc_dec": 1300}
+
+
+def table_share(nbytes: int, sms: int, kind: str) -> float:
+    """The part of a bulk call's blocks that goes through table lookups."""
+    cta = nbytes // 512 // sms
+    spans = cta // CHUNKS_PER_SPAN[kind] if kind in CHUNKS_PER_SPAN else 0
+    return 1.0 - 128 * spans / max(cta, 1)
+
+
 ALU_LANE_OPS_PER_CLK_SM = 64  # LOP3 / PRMT / SHF issue rate of one SM, measured on the GB300
 BITSLICE_SOURCES = ("aes_device.cuh", "bitslice_device.cuh", "kgpu_bitslice.cu", "sbox_circuit.cuh", "kgpu_bitslice.h")
 
@@ -1008,9 +1022,11 @@ def run_kgpu(args):
     achieved_hbm = hbm_bytes / launch_s / 1e9
     hbm_peak = peaks["hbm_gbs"] if peaks else 6800.0
     # shared-memory lookups: Nr = 14 rounds x 16 lookups per 16-B block, plus
-    # one tweak block per 4096-B sector (257 cipher blocks per 256 data blocks)
+    # one tweak block per 4096-B sector (257 cipher blocks per 256 data blocks),
+    # for the blocks that are not enciphered on bit-planes
     nblocks = nbytes // 16
-    lookups = 14 * 16 * nblocks * (257 / 256)
+    share = table_share(nbytes, props.multi_processor_count, "aes256_xts_enc")
+    lookups = 14 * 16 * nblocks * (257 / 256) * share
     smem_bytes = lookups * 4
     sm_mhz = clocks["sm_mhz"] or (peaks or {}).get("sm_max_mhz", 2070.0)
     smem_peak = props.multi_processor_count * SMEM_BYTES_PER_CLK_SM * sm_mhz * 1e6 / 1e9
@@ -1019,7 +1035,7 @@ def run_kgpu(args):
     roofline = {"bound": "smem", "achieved": achieved_smem, "peak": smem_peak, "unit": "GB/s",
                 "frac": achieved_smem / smem_peak, "traffic": traffic,
                 "peak_source": f"{props.multi_processor_count} SMs x 128 B/clk x {sm_mhz:.0f} MHz",
-                "kernel": "bulk_kernel<14,enc,xts>", "launch_ms": launch_s * 1e3}
+                "kernel": ("mixed" if share < 1 else "bulk") + "_kernel<14,enc,xts>", "launch_ms": launch_s * 1e3}
     if bitsliced:
         # ALU-bound: lane-operations of the ALU pipe per block (counted once with
         # ncu on this kernel) x blocks, against SMs x 64 lane-ops/clk x clock
@@ -1072,7 +1088,8 @@ def run_kgpu(args):
         specs.append(("aes128_xts_enc_4k_bitsliced",
                       lambda: ctx.xts_crypt_bitsliced(k128, 0, src, dst, SECTOR, 0, stream)))
         # shared-memory lookups per 16-byte block of each table mode: Nr x 16,
-        # times (1 + 1/blocks per unit) for the XTS tweak; the bitsliced modes
+        # times (1 + 1/blocks per unit) for the XTS tweak, for the blocks that go
+        # through the tables; the bitsliced modes
         # do no lookups (their bound is the ALU, see --variant bitsliced)
         lookups = {"aes256_xts_dec_4k": 14 * 16 * 257 / 256, "aes256_xts_enc_512": 14 * 16 * 33 / 32,
                    "aes128_xts_enc_4k": 10 * 16 * 257 / 256, "aes128_xts_dec_4k": 10 * 16 * 257 / 256,
@@ -1082,7 +1099,8 @@ def run_kgpu(args):
             t = time_op(fn, 20, stream)
             extra[name] = {"GB/s": GIB / t / 1e9, "ms": t * 1e3}
             if name in lookups:
-                bound = smem_bound_clk / (lookups[name] * 4) * 16 / 1e9
+                part = table_share(GIB, props.multi_processor_count, "_".join(name.split("_")[:3]))
+                bound = smem_bound_clk / (lookups[name] * part * 4) * 16 / 1e9
                 extra[name]["smem_bound_GB/s"] = bound
                 extra[name]["frac_of_smem_bound"] = GIB / t / 1e9 / bound
         emit("extra", {"modes": extra})
