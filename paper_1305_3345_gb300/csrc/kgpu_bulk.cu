@@ -87,7 +87,10 @@ __device__ __forceinline__ void xor4(uint4& v, uint32_t a, uint32_t b, uint32_t 
 // visible.  Every CTA waits, so a launch never completes before the one it
 // follows.  GPU time of back-to-back calls without and with it: 4 KiB of
 // AES-256-XTS 7.2 / 4.4 us, 1 MiB 8.2 / 5.5, 16 MiB 30.8 / 28.4, 64 MiB of
-// AES-128-CBC decryption 81.9 / 77.5.
+// AES-128-CBC decryption 81.9 / 77.5.  A waiting CTA keeps its SM from other
+// streams, so CBC encryption, whose chains take 100 us and more, lets the next
+// launch start only when its first warps are at their end (10,000 mixed requests
+// of 4 KiB to 8 MiB, one launch each on eight streams: 96 -> 163 GB/s).
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -505,7 +508,6 @@ template <int NR>
 __global__ void __launch_bounds__(kBulkThreads, 1) cbc_enc_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
-    next_may_start();
     fill_enc(smem);
     wait_for_previous();
     __syncthreads();
@@ -541,6 +543,7 @@ __global__ void __launch_bounds__(kBulkThreads, 1) cbc_enc_kernel(const __grid_c
             if (valid) out[i] = x;
         }
     }
+    if (threadIdx.x < 32) next_may_start();
 }
 
 
@@ -560,7 +563,6 @@ template <int NR, int LANES>
 __global__ void __launch_bounds__(kCbcSplitThreads, 1) cbc_enc_split_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
-    next_may_start();
     fill_enc(smem);
     wait_for_previous();
     constexpr int kCols = 4 / LANES;              // columns per lane
@@ -601,7 +603,9 @@ __global__ void __launch_bounds__(kCbcSplitThreads, 1) cbc_enc_split_kernel(cons
         // the chain is sequential, so plaintext is fetched four blocks ahead
 #pragma unroll
         for (uint32_t i = 0; i < 4; i++) fetch(in + (size_t)LANES * i, valid && i < bpp, q[i]);
+        const uint32_t late = threadIdx.x < 32 && g + total_warps() >= ngroups ? max(bpp, 8u) - 8u : bpp;
         for (uint32_t i = 0; i < bpp; ++i) {
+            if (i == late) next_may_start();
 #pragma unroll
             for (int h = 0; h < kCols; h++) {
                 s[h] = x[h] ^ q[0][h] ^ k[0][h];
@@ -653,7 +657,6 @@ template <int NR>
 __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_staged_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
-    next_may_start();
     fill_enc(smem);
     wait_for_previous();
     __syncthreads();
@@ -706,6 +709,7 @@ __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_staged_kernel
             }
         }
     }
+    if (warp == 0) next_may_start();
 }
 
 // ---------------------------------------------------------------------------
@@ -762,7 +766,6 @@ template <int NR>
 __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_tma_kernel(const __grid_constant__ CbcTmaParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
-    next_may_start();
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
     // kSmemBase + kSmemEnc + warp * 4096: 1024-byte aligned in the shared
@@ -819,6 +822,7 @@ __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_tma_kernel(co
             }
         }
     }
+    if (warp == 0) next_may_start();
     if (!ok && lane == 0) {
         atomicAdd(&g_bulk_wait_timeouts, 1u);
         tile_wait(bar, parity);  // the load still in flight, bounded
@@ -1449,8 +1453,13 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
     if (lanes > 1) {
         auto fn = cbc_enc_split_fn(nr, lanes);
         if (!fn) return cudaErrorInvalidValue;
+        // Two warps share an SM before the next is taken, which costs a chain
+        // nothing and leaves the other SMs to other streams: 4,000 requests of 4
+        // KiB to 8 MiB on eight streams run at 46 GB/s with a warp per SM, 67
+        // with two and 80 with four, 256 pages with AES-256 take 138, 138 and
+        // 140 us.
         const uint64_t teams = (p.npages + 32 / lanes - 1) / (32 / lanes);
-        return launch(fn, (int)std::min<uint64_t>(teams, sms), kCbcSplitThreads, kSmemEnc, s, p);
+        return launch(fn, (int)std::min<uint64_t>((teams + 1) / 2, sms), kCbcSplitThreads, kSmemEnc, s, p);
     }
     // The tensor tiles take a seventh of the staging traffic off the
     // shared-memory path, which pays once that path is the bound: from 12
