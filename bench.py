@@ -130,7 +130,8 @@ class ClockSampler:
 # The sources the bulk XTS kernel is compiled from (its kernels, the device
 # cipher and its parameter structs); a traffic record is valid only for the
 # kernel built from exactly these bytes.
-BULK_KERNEL_SOURCES = ("aes_device.cuh", "bitslice_device.cuh", "kgpu_bulk.cu", "kgpu_bulk.h", "sbox_circuit.cuh")
+BULK_KERNEL_SOURCES = ("aes_device.cuh", "bitslice_device.cuh", "gf128_jump.cuh", "kgpu_bulk.cu", "kgpu_bulk.h",
+                       "sbox_circuit.cuh")
 
 
 def csrc_hash() -> str:
@@ -170,7 +171,8 @@ def table_share(nbytes: int, sms: int, kind: str) -> float:
 
 
 ALU_LANE_OPS_PER_CLK_SM = 64  # LOP3 / PRMT / SHF issue rate of one SM, measured on the GB300
-BITSLICE_SOURCES = ("aes_device.cuh", "bitslice_device.cuh", "kgpu_bitslice.cu", "sbox_circuit.cuh", "kgpu_bitslice.h")
+BITSLICE_SOURCES = ("aes_device.cuh", "bitslice_device.cuh", "gf128_jump.cuh", "kgpu_bitslice.cu", "sbox_circuit.cuh",
+                    "kgpu_bitslice.h")
 
 
 def bitslice_hash() -> str:

@@ -1,8 +1,8 @@
 // Parameter blocks and launch entry points of the bulk kernels (kgpu_bulk.cu):
 // one kernel per mode, direction and key size, for the per-call transforms.
 // Kept apart from the batched and serving formats so that the bulk kernels'
-// sources are exactly aes_device.cuh, bitslice_device.cuh, sbox_circuit.cuh,
-// kgpu_bulk.cu and this header.
+// sources are exactly aes_device.cuh, bitslice_device.cuh, gf128_jump.cuh,
+// sbox_circuit.cuh, kgpu_bulk.cu and this header.
 #pragma once
 #include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
