@@ -647,13 +647,18 @@ __global__ void __launch_bounds__(kCbcSplitThreads, 1) cbc_enc_split_kernel(cons
 // and write their own chains there.  Used when a page is a multiple of 8
 // blocks (128 B).  The next 8 blocks are fetched into registers while the
 // current ones are enciphered.
+//
+// PERMUTE: calls over the host link whose time is a chain's latency build their
+// addresses by byte permutes, which take less of it (64 pages of 64 KiB, AES-128:
+// 2,386 us by dp2a, 2,306 this way).
 // ---------------------------------------------------------------------------
 constexpr int kStageBlocks = 8;
+static_assert(kStageBlocks == kLineBlocks, "a staged chunk is a 128-byte line");
 constexpr int kStageRow = kStageBlocks * 16 + 16;  // one page's 8 blocks, padded against bank conflicts
 constexpr int kStageWarpBytes = 32 * kStageRow;
 static_assert(kStageWarpBytes == kStageWarpSmem, "staging area size");
 
-template <int NR>
+template <int NR, bool PERMUTE>
 __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_staged_kernel(const __grid_constant__ CbcParams p) {
     extern __shared__ __align__(128) char smem[];
     if (!smem_layout_ok(smem)) return;
@@ -663,7 +668,7 @@ __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_staged_kernel
 
     const uint32_t lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5;
-    const Rep4 T{lane * 4u, lane * 4u + 128u};
+    const Rep4Tables<PERMUTE> T{lane * 4u, lane * 4u + 128u};
     const ParamKey K{p.rk};
     const uint32_t bpp = p.bpp;
     const uint32_t nchunks = bpp / kStageBlocks;
@@ -1190,11 +1195,11 @@ KernelFn<CbcParams> cbc_enc_split_fn(int nr, int lanes) {
     }
 }
 
-KernelFn<CbcParams> cbc_enc_staged_fn(int nr) {
+KernelFn<CbcParams> cbc_enc_staged_fn(int nr, bool permute) {
     switch (nr) {
-        case 10: return cbc_enc_staged_kernel<10>;
-        case 12: return cbc_enc_staged_kernel<12>;
-        case 14: return cbc_enc_staged_kernel<14>;
+        case 10: return permute ? cbc_enc_staged_kernel<10, true> : cbc_enc_staged_kernel<10, false>;
+        case 12: return permute ? cbc_enc_staged_kernel<12, true> : cbc_enc_staged_kernel<12, false>;
+        case 14: return permute ? cbc_enc_staged_kernel<14, true> : cbc_enc_staged_kernel<14, false>;
         default: return nullptr;
     }
 }
@@ -1280,9 +1285,11 @@ cudaError_t configure_kernels() {
                                      (int)kSmemEnc);
             if (e != cudaSuccess) return e;
         }
-        e = cudaFuncSetAttribute(cbc_enc_staged_fn(nr), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemEncStaged);
-        if (e != cudaSuccess) return e;
+        for (bool permute : {false, true}) {
+            e = cudaFuncSetAttribute(cbc_enc_staged_fn(nr, permute), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kSmemEncStaged);
+            if (e != cudaSuccess) return e;
+        }
         e = cudaFuncSetAttribute(cbc_enc_tma_fn(nr), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemEncTma);
         if (e != cudaSuccess) return e;
         for (int dir = 0; dir < 2; dir++) {
@@ -1441,15 +1448,8 @@ bool page_tile_maps(CbcTmaParams* t, const CbcParams& p) {
 }
 
 cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t s) {
-    // Few pages are a chain's latency, which two or four lanes per page
-    // shorten; many are the lookups' rate, which one lane per page uses best.
-    // 4-KiB pages, AES-128, one / two / four lanes: 8 pages per SM 145 / 107 /
-    // 103 us, 32 pages 145 / 109 / 107, 64 pages 147 / 121 / 121, 128 pages 153
-    // / 152 / 180, 160 pages 206 / 182 / 288, 192 pages 208 / 207 / 295, 224
-    // pages 215 / 248 / 316.  Pages that cannot be staged cross later (4112 B,
-    // AES-256: 224 pages 299 / 286, 256 pages 306 / 309).
     const uint64_t sms = (uint64_t)(num_sms > 0 ? num_sms : 1);
-    const int lanes = p.npages <= 32 * sms ? 4 : p.npages <= (p.bpp % kStageBlocks ? 240 : 192) * sms ? 2 : 1;
+    const int lanes = cbc_enc_lanes(p.npages, p.bpp, nr, sms, p.link != 0);
     if (lanes > 1) {
         auto fn = cbc_enc_split_fn(nr, lanes);
         if (!fn) return cudaErrorInvalidValue;
@@ -1483,7 +1483,7 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
         }
     }
     if (p.bpp % kStageBlocks == 0) {
-        auto fn = cbc_enc_staged_fn(nr);
+        auto fn = cbc_enc_staged_fn(nr, p.npages <= 192 * sms);
         if (!fn) return cudaErrorInvalidValue;
         const int grid = (int)(groups < (uint64_t)num_sms ? (groups ? groups : 1) : num_sms);
         const int warps = cbc_enc_staged_warps(groups, num_sms);

@@ -142,6 +142,33 @@ struct CtsParams {
     uint32_t tk[kMaxRoundKeyWords];
 };
 
+// ---------------------------------------------------------------------------
+// Which form a call takes, from its sizes alone.
+// ---------------------------------------------------------------------------
+
+constexpr uint32_t kLineBlocks = 8;  // blocks in a 128-byte line
+
+// Lanes that share a page's chain in CBC encryption.  Few pages are a chain's
+// latency, which two or four lanes per page shorten; many are the lookups'
+// rate, which one lane per page uses best.  4-KiB pages, AES-128, one / two /
+// four lanes: 8 pages per SM 145 / 107 / 103 us, 32 pages 145 / 109 / 107, 64
+// pages 147 / 121 / 121, 128 pages 153 / 152 / 180, 160 pages 206 / 182 / 288,
+// 192 pages 208 / 207 / 295, 224 pages 215 / 248 / 316.  Pages that cannot be
+// staged cross later (4112 B, AES-256: 224 pages 299 / 286, 256 pages 306 / 309).
+//
+// Shared lanes move 16 bytes a page at a time.  Over the host link that wins
+// only for a few pages; from there whole lines, which one lane per page moves
+// staged, are several times as fast.  kgpu_crypt on registered 4-KiB pages,
+// shared / staged lanes: AES-128 8 pages 142 / 159 us, 64 pages 144-163 / 159,
+// 1,024 pages 288 / 160, 16,384 pages 1,984 / 510; AES-192 128 pages 172 / 182,
+// 384 pages 192 / 183; AES-256 256 pages 182 / 206, 1,024 pages 288 / 208.
+inline int cbc_enc_lanes(uint64_t npages, uint32_t bpp, int nr, uint64_t sms, bool link) {
+    const bool lines = bpp % kLineBlocks == 0;
+    if (link && lines && npages > (nr == 10 ? 32u : nr == 12 ? 128u : 256u)) return 1;
+    if (npages <= 32 * sms) return 4;
+    return npages <= (lines ? 192 : 240) * sms ? 2 : 1;
+}
+
 cudaError_t launch_xts(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_ecb(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);

@@ -1,0 +1,21 @@
+// The launch rules of the bulk kernels (kgpu_bulk.h), on the CPU.  Reads lines
+//   "e npages bpp nr sms link" -> prints cbc_enc_lanes
+#include <cstdio>
+
+#include "kgpu_bulk.h"
+
+int main() {
+    char kind[2];
+    while (std::scanf("%1s", kind) == 1) {
+        if (kind[0] == 'e') {
+            unsigned long long npages, sms;
+            unsigned bpp;
+            int nr, link;
+            if (std::scanf("%llu %u %d %llu %d", &npages, &bpp, &nr, &sms, &link) != 5) return 2;
+            std::printf("%d\n", kgpu::cbc_enc_lanes(npages, bpp, nr, sms, link != 0));
+        } else {
+            return 2;
+        }
+    }
+    return 0;
+}

@@ -1,0 +1,52 @@
+"""Which form a bulk call takes, decided by the library from its sizes, on the
+CPU through a small C++ harness (tests/bulk_rules_check.cc): every form gives
+the same bytes, so the tests of results cannot tell which one ran."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def ask(tmp_path_factory):
+    cxx = shutil.which("g++")
+    cuda_inc = "/usr/local/cuda/include"
+    if not cxx or not os.path.exists(os.path.join(cuda_inc, "cuda_runtime.h")):
+        pytest.skip("g++ or the CUDA headers are not available")
+    exe = str(tmp_path_factory.mktemp("rules") / "bulk_rules_check")
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I", os.path.join(ROOT, "paper_1305_3345_gb300", "csrc"), "-I", cuda_inc,
+                    os.path.join(HERE, "bulk_rules_check.cc"), "-o", exe], check=True)
+
+    def run(kind, *args):
+        line = " ".join(map(str, (kind, *args))) + "\n"
+        return int(subprocess.run([exe], input=line, capture_output=True, text=True, check=True).stdout)
+    return run
+
+
+@pytest.mark.parametrize("bpp", [1, 8, 256, 257, 4096])
+def test_cbc_encryption_of_device_pages(ask, bpp):
+    most = 192 if bpp % 8 == 0 else 240
+    for nr in (10, 12, 14):
+        assert ask("e", 1, bpp, nr, SMS, 0) == 4
+        assert ask("e", 32 * SMS, bpp, nr, SMS, 0) == 4
+        assert ask("e", 32 * SMS + 1, bpp, nr, SMS, 0) == 2
+        assert ask("e", most * SMS, bpp, nr, SMS, 0) == 2
+        assert ask("e", most * SMS + 1, bpp, nr, SMS, 0) == 1
+
+
+@pytest.mark.parametrize("nr,few", [(10, 32), (12, 128), (14, 256)])
+def test_cbc_encryption_over_the_link_moves_whole_lines(ask, nr, few):
+    """Pages in whole 128-byte lines are staged, but for a few pages; shared
+    lanes would move 16 bytes a page at a time."""
+    for bpp in (8, 32, 256, 4096):
+        assert ask("e", few, bpp, nr, SMS, 1) == 4
+        for n in (few + 1, 4096, 32 * SMS + 1, 192 * SMS):
+            assert ask("e", n, bpp, nr, SMS, 1) == 1
+    # what cannot be staged is as on the device
+    assert ask("e", 32 * SMS, 257, nr, SMS, 1) == 4
+    assert ask("e", 240 * SMS, 257, nr, SMS, 1) == 2
