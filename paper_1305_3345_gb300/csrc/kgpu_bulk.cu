@@ -1453,13 +1453,8 @@ cudaError_t launch_cbc_enc(const CbcParams& p, int nr, int num_sms, cudaStream_t
     if (lanes > 1) {
         auto fn = cbc_enc_split_fn(nr, lanes);
         if (!fn) return cudaErrorInvalidValue;
-        // Two warps share an SM before the next is taken, which costs a chain
-        // nothing and leaves the other SMs to other streams: 4,000 requests of 4
-        // KiB to 8 MiB on eight streams run at 46 GB/s with a warp per SM, 67
-        // with two and 80 with four, 256 pages with AES-256 take 138, 138 and
-        // 140 us.
         const uint64_t teams = (p.npages + 32 / lanes - 1) / (32 / lanes);
-        return launch(fn, (int)std::min<uint64_t>((teams + 1) / 2, sms), kCbcSplitThreads, kSmemEnc, s, p);
+        return launch(fn, (int)cbc_enc_split_ctas(teams, sms), kCbcSplitThreads, kSmemEnc, s, p);
     }
     // The tensor tiles take a seventh of the staging traffic off the
     // shared-memory path, which pays once that path is the bound: from 12

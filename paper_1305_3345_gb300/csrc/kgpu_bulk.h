@@ -169,6 +169,19 @@ inline int cbc_enc_lanes(uint64_t npages, uint32_t bpp, int nr, uint64_t sms, bo
     return npages <= (lines ? 192 : 240) * sms ? 2 : 1;
 }
 
+// CTAs for teams of one warp each that split chains over lanes.  Two warps share
+// an SM before the next is taken, which costs a chain nothing; past an eighth
+// of the SMs three do, so that calls on several streams run beside each other
+// (4 MiB of AES-128 on eight streams: two warps an SM 47.7 us a call, three
+// 33.4, a warp a page group without split chains 32.8).  A call by itself takes
+// 102.3 us with three, 101.7 with two and 103.7 with four.
+inline uint64_t cbc_enc_split_ctas(uint64_t teams, uint64_t sms) {
+    const uint64_t two = (teams + 1) / 2, three = (teams + 2) / 3;
+    const uint64_t eighth = sms / 8;
+    const uint64_t n = two <= eighth ? two : three > eighth ? three : eighth;
+    return n < 1 ? 1 : n < sms ? n : sms;
+}
+
 cudaError_t launch_xts(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_ecb(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);

@@ -1,5 +1,6 @@
 // The launch rules of the bulk kernels (kgpu_bulk.h), on the CPU.  Reads lines
 //   "e npages bpp nr sms link" -> prints cbc_enc_lanes
+//   "s teams sms"               -> prints cbc_enc_split_ctas
 #include <cstdio>
 
 #include "kgpu_bulk.h"
@@ -13,6 +14,10 @@ int main() {
             int nr, link;
             if (std::scanf("%llu %u %d %llu %d", &npages, &bpp, &nr, &sms, &link) != 5) return 2;
             std::printf("%d\n", kgpu::cbc_enc_lanes(npages, bpp, nr, sms, link != 0));
+        } else if (kind[0] == 's') {
+            unsigned long long teams, sms;
+            if (std::scanf("%llu %llu", &teams, &sms) != 2) return 2;
+            std::printf("%llu\n", (unsigned long long)kgpu::cbc_enc_split_ctas(teams, sms));
         } else {
             return 2;
         }

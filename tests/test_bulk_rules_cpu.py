@@ -50,3 +50,20 @@ def test_cbc_encryption_over_the_link_moves_whole_lines(ask, nr, few):
     # what cannot be staged is as on the device
     assert ask("e", 32 * SMS, 257, nr, SMS, 1) == 4
     assert ask("e", 240 * SMS, 257, nr, SMS, 1) == 2
+
+
+def test_split_chains_leave_sms_to_other_streams(ask):
+    """At least one CTA, never more than SMs or 16 warps to one, two warps an SM
+    while that takes an eighth of the SMs, at most three further on."""
+    last = 0
+    for teams in list(range(1, 400)) + [1216, 1824, 1825, 2432]:
+        n = ask("s", teams, SMS)
+        assert 1 <= n <= SMS and n >= last and n * 16 >= teams
+        last = n
+        if teams <= 2 * (SMS // 8):
+            assert n == (teams + 1) // 2
+        elif teams <= 3 * SMS:
+            assert n == max(SMS // 8, (teams + 2) // 3)
+        else:
+            assert n == SMS
+    assert ask("s", 5, 1) == 1 and ask("s", 5, 7) <= 2
