@@ -455,15 +455,6 @@ int kgpu_bulk_wait_timeouts(kgpu_ctx* ctx, uint32_t* count) {
     return KGPU_OK;
 }
 
-// SMs for a launch whose pages cross the host link.  A quarter of them enciphers
-// at up to 179 GB/s, above the 171 GB/s that the link moves in both directions,
-// and leaves the others free: 8 MiB took 76 us on 152 SMs, 75 on 76 and 70 on
-// 38, 64 MiB 435 / 466 / 427, 1 GiB 6,420 / 7,147 / 6,521.  Units of less than
-// 512 bytes spend more lookups on tweaks and keep the whole device.
-static int link_sms(const kgpu_ctx* ctx, const BulkParams& p) {
-    return p.bps >= 32 ? (ctx->num_sms + 3) / 4 : ctx->num_sms;
-}
-
 int kgpu_aes_xts_crypt_host(kgpu_ctx* ctx, kgpu_key key, int dir, const void* src, void* dst, size_t len,
                             size_t du_size, uint64_t first_sector, size_t chunk_bytes) {
     int rc = xts_args(ctx, dir, len, du_size, first_sector);
@@ -498,7 +489,7 @@ int kgpu_aes_xts_crypt_host(kgpu_ctx* ctx, kgpu_key key, int dir, const void* sr
         fill_bulk(&p, k, dir, reinterpret_cast<const void*>(hsrc), reinterpret_cast<void*>(hdst), len, du_size,
                   first_sector);
         p.link = 1;
-        cudaError_t e = launch_xts(p, k.nr, dir, link_sms(ctx, p), ctx->hs[0]);
+        cudaError_t e = launch_xts(p, k.nr, dir, link_sms(ctx->num_sms, p.bps, len), ctx->hs[0]);
         cudaError_t e2 = cudaStreamSynchronize(ctx->hs[0]);
         return from_cuda(e != cudaSuccess ? e : e2);
     }

@@ -182,6 +182,22 @@ inline uint64_t cbc_enc_split_ctas(uint64_t teams, uint64_t sms) {
     return n < 1 ? 1 : n < sms ? n : sms;
 }
 
+// SMs for a launch whose pages cross the host link.  A quarter of them enciphers
+// about as fast as the link moves pages in both directions (171 GB/s), leaves
+// the others free and, for short calls, is the faster: AES-256-XTS in 4-KiB units
+// on 38 / 114 / 152 SMs 4 MiB 54 / 59 / 61 us, 16 MiB 130 / 136 / 138, 64 MiB 434
+// / 439 / 442.  Long calls run into the lookups there, the sooner the more of
+// them go to tweaks, and want three quarters: 128 MiB 844 / 843 / 852, 1 GiB 6,604
+// / 6,516 / 6,566; 512-byte units 32 MiB 240 / 236 / 240, 64 MiB 455 / 438 / 444, 1
+// GiB 6,831 / 6,533 / 6,576.  (Half the SMs are slower than either at 4-KiB units,
+// 7,090 at 1 GiB, in every run; why is not known.)  Units of less than 512 bytes
+// keep the whole device.
+inline int link_sms(int num_sms, uint32_t unit_blocks, uint64_t bytes) {
+    if (unit_blocks < 32) return num_sms;
+    const uint64_t most = (unit_blocks >= 128 ? 96ull : 48ull) << 20;
+    return bytes <= most ? (num_sms + 3) / 4 : (3 * num_sms + 3) / 4;
+}
+
 cudaError_t launch_xts(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_ecb(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);

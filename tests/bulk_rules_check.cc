@@ -1,6 +1,7 @@
 // The launch rules of the bulk kernels (kgpu_bulk.h), on the CPU.  Reads lines
 //   "e npages bpp nr sms link" -> prints cbc_enc_lanes
 //   "s teams sms"               -> prints cbc_enc_split_ctas
+//   "l sms unit_blocks bytes"   -> prints link_sms
 #include <cstdio>
 
 #include "kgpu_bulk.h"
@@ -18,6 +19,12 @@ int main() {
             unsigned long long teams, sms;
             if (std::scanf("%llu %llu", &teams, &sms) != 2) return 2;
             std::printf("%llu\n", (unsigned long long)kgpu::cbc_enc_split_ctas(teams, sms));
+        } else if (kind[0] == 'l') {
+            int sms;
+            unsigned unit;
+            unsigned long long bytes;
+            if (std::scanf("%d %u %llu", &sms, &unit, &bytes) != 3) return 2;
+            std::printf("%d\n", kgpu::link_sms(sms, unit, bytes));
         } else {
             return 2;
         }

@@ -67,3 +67,14 @@ def test_split_chains_leave_sms_to_other_streams(ask):
         else:
             assert n == SMS
     assert ask("s", 5, 1) == 1 and ask("s", 5, 7) <= 2
+
+
+def test_sms_for_pages_over_the_link(ask):
+    """A quarter of the SMs for short calls, three quarters for long ones, all
+    for units under 512 bytes."""
+    mib = 1 << 20
+    for unit, most in ((32, 48), (64, 48), (128, 96), (256, 96), (1 << 20, 96)):
+        assert ask("l", SMS, unit, 16) == ask("l", SMS, unit, most * mib) == 38
+        assert ask("l", SMS, unit, most * mib + 1) == ask("l", SMS, unit, 1024 * mib) == 114
+        assert ask("l", 1, unit, mib) == ask("l", 1, unit, 1024 * mib) == 1
+    assert ask("l", SMS, 31, mib) == ask("l", SMS, 1, 1024 * mib) == SMS

@@ -50,3 +50,27 @@ def test_cbc_encryption_over_the_link_is_link_bound(ctx):
     finally:
         hp.close()
         ctx.delkey(kh)
+
+
+@pytest.mark.parametrize("bits,dir,du,mib", [(128, 1, 512, 48), (256, 0, 4096, 96), (256, 1, 528, 48)])
+def test_host_call_at_the_line_between_sm_counts(ctx, bits, dir, du, mib):
+    """Registered pages just up to and past the size from which more SMs run."""
+    import torch
+    key = w.xts_key(93, bits)
+    kh = ctx.setkey(key, True)
+    units = (mib << 20) // du + 1
+    data = w.seeded_bytes(93 + du, w.STREAM_DATA, du * units)
+    src = torch.from_numpy(data.copy()).pin_memory()
+    dst = torch.zeros(du * units, dtype=torch.uint8).pin_memory()
+    ref = oracle.xts(key, dir, data, du, 9)
+    ctx.host_register(src)
+    ctx.host_register(dst)
+    try:
+        for n in (units - 1, units):
+            dst.zero_()
+            ctx.xts_crypt_host(kh, dir, src[:n * du], dst[:n * du], du, 9)
+            assert np.array_equal(dst.numpy()[:n * du], ref[:n * du]), (bits, dir, du, n)
+    finally:
+        ctx.host_unregister(src)
+        ctx.host_unregister(dst)
+        ctx.delkey(kh)
