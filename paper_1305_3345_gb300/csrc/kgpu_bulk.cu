@@ -1359,6 +1359,7 @@ cudaError_t launch_cbc_dec(const CbcParams& p, int nr, int num_sms, cudaStream_t
     auto fn = cbc_fn(nr, false);
     if (!fn) return cudaErrorInvalidValue;
     CbcParams q = p;
+    num_sms = cbc_dec_sms(num_sms, p.bpp, p.npages * p.bpp * 16, p.link != 0);
     const bool in_place = p.src == p.dst;
     const uint64_t items = in_place ? p.npages : (p.npages * p.bpp + 31) / 32;
     const int grid = in_place ? (int)std::min<uint64_t>(items, num_sms) : grid_for_chunks(items, num_sms);

@@ -198,6 +198,14 @@ inline int link_sms(int num_sms, uint32_t unit_blocks, uint64_t bytes) {
     return bytes <= most ? (num_sms + 3) / 4 : (3 * num_sms + 3) / 4;
 }
 
+// SMs for CBC decryption: over the host link, from the sizes where a call that
+// takes them all is bound by it, as for XTS (registered 4-KiB pages, AES-128, 152
+// / 38 SMs: 1 MiB 24.5 / 24.3 us, AES-256 24.6 / 25.9; 2 MiB 34.4 / 31.6; 4 MiB
+// 50.8 / 44.8; 8 MiB 77.3 / 71.2).
+inline int cbc_dec_sms(int num_sms, uint32_t bpp, uint64_t bytes, bool link) {
+    return link && bytes >= (2ull << 20) ? link_sms(num_sms, bpp, bytes) : num_sms;
+}
+
 cudaError_t launch_xts(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_xts_cts(const CtsParams& p, int nr, int dir, int num_sms, cudaStream_t s);
 cudaError_t launch_ecb(const BulkParams& p, int nr, int dir, int num_sms, cudaStream_t s);

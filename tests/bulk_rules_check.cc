@@ -2,6 +2,7 @@
 //   "e npages bpp nr sms link" -> prints cbc_enc_lanes
 //   "s teams sms"               -> prints cbc_enc_split_ctas
 //   "l sms unit_blocks bytes"   -> prints link_sms
+//   "d sms bpp bytes link"      -> prints cbc_dec_sms
 #include <cstdio>
 
 #include "kgpu_bulk.h"
@@ -25,6 +26,12 @@ int main() {
             unsigned long long bytes;
             if (std::scanf("%d %u %llu", &sms, &unit, &bytes) != 3) return 2;
             std::printf("%d\n", kgpu::link_sms(sms, unit, bytes));
+        } else if (kind[0] == 'd') {
+            int sms, link;
+            unsigned bpp;
+            unsigned long long bytes;
+            if (std::scanf("%d %u %llu %d", &sms, &bpp, &bytes, &link) != 4) return 2;
+            std::printf("%d\n", kgpu::cbc_dec_sms(sms, bpp, bytes, link != 0));
         } else {
             return 2;
         }

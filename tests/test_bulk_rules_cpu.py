@@ -78,3 +78,13 @@ def test_sms_for_pages_over_the_link(ask):
         assert ask("l", SMS, unit, most * mib + 1) == ask("l", SMS, unit, 1024 * mib) == 114
         assert ask("l", 1, unit, mib) == ask("l", 1, unit, 1024 * mib) == 1
     assert ask("l", SMS, 31, mib) == ask("l", SMS, 1, 1024 * mib) == SMS
+
+
+def test_sms_for_cbc_decryption(ask):
+    mib = 1 << 20
+    for bytes_ in (4096, 4 * mib, 1024 * mib):
+        assert ask("d", SMS, 256, bytes_, 0) == SMS
+    assert ask("d", SMS, 256, 2 * mib - 4096, 1) == SMS
+    assert ask("d", SMS, 256, 2 * mib, 1) == ask("d", SMS, 32, 48 * mib, 1) == 38
+    assert ask("d", SMS, 32, 49 * mib, 1) == ask("d", SMS, 256, 97 * mib, 1) == 114
+    assert ask("d", SMS, 16, 64 * mib, 1) == SMS

@@ -74,3 +74,21 @@ def test_host_call_at_the_line_between_sm_counts(ctx, bits, dir, du, mib):
         ctx.host_unregister(src)
         ctx.host_unregister(dst)
         ctx.delkey(kh)
+
+
+@pytest.mark.parametrize("bits,unit,pages", [(128, 4096, 511), (256, 4096, 513), (192, 528, 9000), (128, 512, 98305)])
+def test_cbc_decryption_over_the_link(ctx, bits, unit, pages):
+    import paper_1305_3345_gb300 as kg
+    key = w.single_key(94, bits)
+    kh = ctx.setkey(key, False)
+    hp = HostPages(ctx, 94 + unit, unit * pages, unit)
+    try:
+        ref = oracle.cbc(key, 1, hp.data, unit, hp.ivs_np[:pages])
+        for out in (hp.dst, hp.src):  # out of place, then in place
+            r = request(kg, kg.MODE_CBC_DEC, kh, hp.src.data_ptr(), out.data_ptr(), unit * pages, unit,
+                        ivs=hp.ivs.data_ptr())
+            assert ctx.crypt(r, kg.DISPATCH_GPU) == (0, kg.DISPATCH_GPU)
+            assert np.array_equal(out.numpy(), ref), (bits, unit, pages)
+    finally:
+        hp.close()
+        ctx.delkey(kh)
