@@ -469,6 +469,25 @@ int make_desc(kgpu_ctx* ctx, const kgpu_request& q, Cache& rc, uint32_t tile_chu
 }
 
 
+constexpr uint32_t kBacklogTileChunks = 64;  // 32 KiB: tiles of requests served under backlog
+
+// Tile size (512-byte chunks) of a served request of nblocks blocks whose caller
+// has set none.  Requests that arrive together are a small backlog of their
+// own: a burst of burst_bytes gets tiles that leave every worker warp at least
+// four, between the default size and the backlog's (a burst of 128 XTS requests,
+// 24 MB: 130 us in 1-KiB tiles, 112 in 2-KiB ones).  Requests on host pages, which
+// the link bounds, keep the default: larger tiles leave it less even work (500
+// XTS requests of 4 KiB to 2 MiB on registered pages 1,138 us in 1-KiB tiles,
+// 1,254 in the burst's; 300 up to 1 MiB 462 / 520), unless they would then have
+// more than the max_tiles that a request may have.
+inline uint32_t burst_tile_chunks(uint32_t chunks, uint64_t nblocks, uint64_t burst_bytes, uint64_t workers,
+                                  bool host, uint64_t max_tiles) {
+    if (host && (nblocks + 31) / 32 <= max_tiles * chunks) return chunks;
+    uint32_t t = chunks;
+    while (t < kBacklogTileChunks && burst_bytes / (512ull * 8 * t) >= workers) t *= 2;
+    return t;
+}
+
 // Tile size (512-byte chunks) of a batch whose caller has set none: 32, or
 // less where the batch then has fewer tiles than the launch has warps, down
 // to the two chunks that a warp enciphers at a time (50 XTS requests of 4 KiB

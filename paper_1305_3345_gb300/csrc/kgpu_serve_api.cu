@@ -267,10 +267,6 @@ struct ReaderGuard {
     ReaderGuard& operator=(const ReaderGuard&) = delete;
 };
 
-// Publish a validated descriptor.  Caller holds serve_mu.
-// Tile size of requests staged while the ring is backed up (512-byte chunks).
-constexpr uint32_t kBacklogTileChunks = 64;  // 32 KiB
-
 // Write one request into the next ring slot, without making it visible to
 // the device yet (commit does that).  Caller holds serve_mu.
 //
@@ -279,7 +275,7 @@ constexpr uint32_t kBacklogTileChunks = 64;  // 32 KiB
 // it gets 32-KiB tiles: per tile the workers claim a position, reload a key
 // schedule and (for XTS) run a 32-unit tweak batch, and on small tiles those
 // costs cap the ring's throughput.  A ring that keeps up keeps the configured
-// (default 2-KiB) tiles and their lower latency, and runs CBC encryption four
+// (default 1-KiB) tiles and their lower latency, and runs CBC encryption four
 // lanes to a page (twice the chain speed, a quarter of the pages per warp;
 // host pages through the warp's scratch area, whole lines at a time).  The
 // check is one load of a completion word, whatever the number of requests in
@@ -291,16 +287,12 @@ bool backlogged(const ServeState& st) {
     return load_acquire(&st.done_seq[seq & (st.nslots - 1)]) < seq + 1;
 }
 
-// Requests that arrive together are a small backlog of their own: a burst of
-// burst_bytes gets tiles that leave every worker warp at least four, between
-// the default size and the backlog's, unless the caller set a size (a burst of
-// 128 XTS requests, 24 MB: 130 us in 1-KiB tiles, 112 in 2-KiB ones).
 int stage(ServeState& st, const ReqDesc& dreq, uint64_t burst_bytes, uint64_t* seq_out) {
     ReqDesc d = dreq;
     if (st.auto_tiles && d.mode != KGPU_MODE_COPY) {
-        uint32_t t = st.tile_chunks;
-        while (t < kBacklogTileChunks && burst_bytes / (512ull * 8 * t) >= st.workers) t *= 2;
-        set_tile_units(d, t);
+        const bool host = (d.flags & (kDescSrcHost | kDescDstHost)) != 0;
+        set_tile_units(d, burst_tile_chunks(st.tile_chunks, d.nblocks, burst_bytes, st.workers, host,
+                                            serve_max_tiles(st.tile_ring)));
     }
     if (backlogged(st)) {
         set_tile_units(d, std::max<uint32_t>(st.tile_chunks, kBacklogTileChunks));
