@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <type_traits>
 #include <mutex>
@@ -1161,15 +1162,28 @@ KernelFn<MixCbcParams> mixed_cbc_dec_fn(int nr) {
 
 size_t mixed_smem(int dir) { return (dir == 0 ? kSmemEnc : kSmemDec) + kMixTweakBytes; }
 
+// The mixed kernels that may be launched, one bit each: those compiled to the
+// register count that the register shares of their warps are drawn from (a
+// share beyond it would wait for ever).  Another compiler may give another
+// count; calls then stay on the table kernels, which take every size.
+std::atomic<uint32_t> g_mixed_usable{0};
+
+constexpr uint32_t mixed_bit(int nr, int dir, bool tweak) { return 1u << ((nr - 10) * 2 + dir * 2 + (tweak ? 1 : 0)); }
+constexpr uint32_t mixed_cbc_dec_bit(int nr) { return 1u << (12 + (nr - 10) / 2); }
+
 template <class P>
-cudaError_t configure_mixed(KernelFn<P> fn, size_t smem) {
+cudaError_t configure_mixed(KernelFn<P> fn, size_t smem, uint32_t bit) {
     if (!fn) return cudaSuccess;
     cudaFuncAttributes attr;
     cudaError_t e = cudaFuncGetAttributes(&attr, fn);
     if (e != cudaSuccess) return e;
-    // what the register shares of its warps are drawn from
-    if (attr.numRegs != kMixLaunchRegs) return cudaErrorInvalidConfiguration;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr.numRegs != kMixLaunchRegs) {
+        g_mixed_usable.fetch_and(~bit);
+        return cudaSuccess;
+    }
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) g_mixed_usable.fetch_or(bit);
+    return e;
 }
 
 void plane_masks(uint32_t* masks, const uint32_t* rk, int nr) {
@@ -1269,11 +1283,11 @@ cudaError_t configure_kernels() {
                 cudaError_t e = cudaFuncSetAttribute(bulk_fn(nr, dir, tw), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)bulk_smem(dir, tw));
                 if (e != cudaSuccess) return e;
-                e = configure_mixed(mixed_fn(nr, dir, tw), mixed_smem(dir));
+                e = configure_mixed(mixed_fn(nr, dir, tw), mixed_smem(dir), mixed_bit(nr, dir, tw));
                 if (e != cudaSuccess) return e;
             }
         }
-        cudaError_t e = configure_mixed(mixed_cbc_dec_fn(nr), kSmemDec);
+        cudaError_t e = configure_mixed(mixed_cbc_dec_fn(nr), kSmemDec, mixed_cbc_dec_bit(nr));
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(cbc_fn(nr, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemEnc);
@@ -1337,7 +1351,9 @@ static cudaError_t launch_bulk(const BulkParams& params, int nr, int dir, bool t
     if (chunks / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     p.cta_chunks = (uint32_t)(chunks / grid);
     p.cta_rest = (uint32_t)(chunks % grid);
-    if (const uint32_t spans = mix_spans(p.cta_chunks, nr, dir, tweak, tweak ? p.bps : 32, p.link != 0)) {
+    const bool usable = (g_mixed_usable.load() & mixed_bit(nr, dir, tweak)) != 0;
+    const uint32_t spans = usable ? mix_spans(p.cta_chunks, nr, dir, tweak, tweak ? p.bps : 32, p.link != 0) : 0;
+    if (spans) {
         MixParams mp;
         mp.b = p;
         mp.spans = spans;
@@ -1366,7 +1382,9 @@ cudaError_t launch_cbc_dec(const CbcParams& p, int nr, int num_sms, cudaStream_t
     if (items / grid >= 0xffffffffull) return cudaErrorInvalidValue;
     q.cta_items = (uint32_t)(items / grid);
     q.cta_rest = (uint32_t)(items % grid);
-    if (const uint32_t spans = in_place ? 0 : mix_spans(q.cta_items, nr, 1, false, p.bpp, p.link != 0)) {
+    const bool usable = !in_place && (g_mixed_usable.load() & mixed_cbc_dec_bit(nr)) != 0;
+    const uint32_t spans = usable ? mix_spans(q.cta_items, nr, 1, false, p.bpp, p.link != 0) : 0;
+    if (spans) {
         MixCbcParams mp;
         mp.c = q;
         mp.spans = spans;
