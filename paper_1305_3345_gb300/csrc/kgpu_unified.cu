@@ -1031,14 +1031,12 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
     const ReqDesc* reqs = reinterpret_cast<const ReqDesc*>(a.buf + batch_desc_offset());
     const uint64_t* tile_start = reinterpret_cast<const uint64_t*>(a.buf + batch_prefix_offset(nreq));
     const uint32_t* order = reinterpret_cast<const uint32_t*>(a.buf + batch_order_offset(nreq));
-    unsigned long long* work = a.next_tile;
-    unsigned long long* fin = a.fin;
-    int* status = a.status;
-    if (!work) {
-        work = reinterpret_cast<unsigned long long*>(a.buf + batch_zeros_offset(nreq));
-        fin = work + 2;
-        status = reinterpret_cast<int*>(fin + nreq);
-    }
+    unsigned long long* const work =
+        a.next_tile ? a.next_tile : reinterpret_cast<unsigned long long*>(a.buf + batch_zeros_offset(nreq));
+    // formed where a tile needs them: held over the loop, the two pointers made
+    // the 1,024-thread variant spill
+    auto fin_words = [&]() { return a.next_tile ? a.fin : work + 2; };
+    auto status_words = [&]() { return a.next_tile ? a.status : reinterpret_cast<int*>(work + 2 + nreq); };
     // Two queues: the CBC-encryption tiles, whose time is a chain's latency,
     // and the others.  The first long_warps warps of every CTA start with the
     // chains, so that these run beside each other and beside other work from
@@ -1078,8 +1076,8 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
         const ReqDesc d = reqs[i];
         const int st = run_tile<false, (THREADS <= 512)>(d, t - tile_start[k], a.keys, a.max_keys, K, cur_sel, cur_gen, stage,
                                                            pool);
-        if (st && lane == 0) status[i] = st;
-        if (fin) {
+        if (st && lane == 0) status_words()[i] = st;
+        if (unsigned long long* fin = fin_words()) {
             // per-request completion: the warp that finishes a request's last
             // tile publishes (tag << 32 | status) to the host-mapped word,
             // after an acq_rel count that orders every warp's tile writes
@@ -1089,7 +1087,7 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
             if (lane == 0) f = atom_add_acq_rel_gpu(&fin[i], 1ull) + 1;
             f = __shfl_sync(0xffffffffu, f, 0);
             if (lane == 0 && f == tile_start[k + 1] - tile_start[k]) {
-                const unsigned int code = (unsigned int)*reinterpret_cast<volatile int*>(&status[i]);
+                const unsigned int code = (unsigned int)*reinterpret_cast<volatile int*>(&status_words()[i]);
                 st_release_sys(&a.done[i], (unsigned long long)hdr->tag << 32 | code);
             }
         }
