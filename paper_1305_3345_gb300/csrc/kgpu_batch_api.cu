@@ -260,7 +260,8 @@ int kgpu_submit(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, kgpu_stream s
     kgpu_tuning t = effective(ctx);
     // CBC encryption of host pages is staged only in the 512-thread kernel
     if (t.threads > 512 && needs_staging(reqs, n)) t.threads = 512;
-    if (!ctx->tune.tile_chunks) t.tile_chunks = default_tile_chunks(reqs, n, (uint64_t)t.ctas * (t.threads / 32));
+    const uint32_t resident = resident_ctas(t.ctas, ctx->num_sms);
+    if (!ctx->tune.tile_chunks) t.tile_chunks = default_tile_chunks(reqs, n, (uint64_t)resident * (t.threads / 32));
     const uint64_t ticket = ++ctx->next_ticket;
     kgpu::BatchSlot& s = ctx->slots[ticket % kBatchSlots];
     // a batch someone waits on (kgpu_poll, kgpu_poll_each) keeps its slot
@@ -280,7 +281,7 @@ int kgpu_submit(kgpu_ctx* ctx, const kgpu_request* reqs, size_t n, kgpu_stream s
     s.issued = false;
     int rc = prepare_slot(ctx, s, n ? n : 1, t);
     if (rc) return rc;
-    rc = pack_batch(ctx, reqs, n, t.tile_chunks, t.ctas, t.threads / 32, s.h_buf, req_status);
+    rc = pack_batch(ctx, reqs, n, t.tile_chunks, resident, t.threads / 32, s.h_buf, req_status);
     if (rc) return rc;
     s.nreq = (uint32_t)n;
     s.gen = ticket;

@@ -88,7 +88,7 @@ struct BatchHeader {
     uint32_t tag;  // low 32 bits of the batch's ticket, in its completion words
     uint64_t long_tiles;  // the CBC-encryption tiles: the first ones in run order
     uint32_t long_warps;  // warps per CTA that start with them
-    uint32_t pad;
+    uint32_t ctas;        // CTAs of the launch that run at once
 };
 
 // Byte layout of a batch on the device: header, descriptors, tile prefix, run order.

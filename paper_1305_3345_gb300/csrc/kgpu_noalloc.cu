@@ -123,8 +123,9 @@ extern "C" int kgpu_submit_noalloc(kgpu_ctx* ctx, const kgpu_request* reqs, size
     const uint32_t ctas = t.ctas ? t.ctas : (uint32_t)ctx->num_sms;
     // CBC encryption of host pages is staged only in the 512-thread kernel
     if (threads > 512 && needs_staging(reqs, n)) threads = 512;
+    const uint32_t resident = resident_ctas(ctas, ctx->num_sms);
     const uint32_t tile_chunks =
-        t.tile_chunks ? t.tile_chunks : default_tile_chunks(reqs, n, (uint64_t)ctas * (threads / 32));
+        t.tile_chunks ? t.tile_chunks : default_tile_chunks(reqs, n, (uint64_t)resident * (threads / 32));
 
     std::lock_guard<std::mutex> lk(g_pack_mu);
     FixedRangeCache cache;
@@ -136,7 +137,7 @@ extern "C" int kgpu_submit_noalloc(kgpu_ctx* ctx, const kgpu_request* reqs, size
         if (r && !first) first = r;
     }
     if (first) return first;
-    plan_batch(g_pack, (uint32_t)n, [](uint32_t) { return false; }, ctas, threads / 32);
+    plan_batch(g_pack, (uint32_t)n, [](uint32_t) { return false; }, resident, threads / 32);
 
     BatchArgs a{};
     a.buf = scratch + kBatchOff;

@@ -1051,8 +1051,8 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
     const uint64_t longs = hdr->long_tiles, shorts = total - longs;
     const uint32_t first_short = hdr->long_warps;
     bool on_long = warp < first_short;
-    if (!on_long && (uint64_t)(warp - first_short) * gridDim.x >= shorts) {
-        if ((uint64_t)warp * gridDim.x >= total) return;  // more warps than tiles
+    if (!on_long && (uint64_t)(warp - first_short) * hdr->ctas >= shorts) {
+        if ((uint64_t)warp * hdr->ctas >= total) return;  // more warps than tiles
         on_long = true;
     }
     bool other = true;  // the other queue has not been tried
@@ -1069,7 +1069,7 @@ __global__ void __launch_bounds__(THREADS, 1) batch_kernel(const __grid_constant
             continue;
         }
         const uint64_t t = on_long ? next : longs + next;
-        const bool ahead = !on_long && next + 2 * (uint64_t)total_warps() < shorts;
+        const bool ahead = !on_long && next + 2 * (uint64_t)(hdr->ctas * (THREADS / 32)) < shorts;
         if (ahead && lane == 0) next = atomicAdd(&work[1], 1ull);
         const uint32_t k = find_request(tile_start, nreq, t);
         const uint32_t i = order[k];
