@@ -158,7 +158,7 @@ def recorded_traffic():
 
 # 512-byte chunks a CTA (one per SM) needs for each span of 32 chunks that each
 # of its four bitsliced warps takes off the tables: the launch rule of the bulk
-# kernels (mix_spans in kgpu_bulk.cu)
+# kernels (mix_spans in kgpu_bulk.h; a CPU test compares the two)
 CHUNKS_PER_SPAN = {"aes256_xts_enc": 1300, "aes128_xts_enc": 1400, "aes256_xts_dec": 1600, "aes128_xts_dec": 1800,
                    "aes128_ecb_enc": 1250, "aes128_cbc_dec": 1300}
 

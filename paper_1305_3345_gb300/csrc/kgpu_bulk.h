@@ -146,6 +146,27 @@ struct CtsParams {
 // Which form a call takes, from its sizes alone.
 // ---------------------------------------------------------------------------
 
+// Spans that each bitsliced warp of a CTA takes from a run of cta_chunks
+// 32-block chunks; 0: the call stays on the tables.  A warp that takes one span
+// too many costs the call up to a span's time, so a span is given for every
+// so many chunks as the table warps encipher meanwhile, rounded down.  1 GiB
+// (13,797 chunks a CTA) of AES-256-XTS by spans per warp: 0 1,584 us, 10 1,475,
+// 11 1,527; of AES-128 0 1,155, 9 1,099, 10 1,160; of ECB, which forms no
+// tweaks, with AES-256 0 1,573, 10 1,443, 11 1,428, with AES-128 9 1,066, 11
+// 1,046; of decryption with AES-256-XTS 0 1,591, 8 1,524, 9 1,540, with AES-128
+// 0 1,165, 7 1,130, 8 1,135; of CBC decryption with AES-256 0 1,616, 10 1,541, 11
+// 1,563, with AES-128 0 1,189, 10 1,121, 11 1,165.  Units under 512 bytes have
+// more tweaks than a span has lanes, and pages that cross the host link are
+// bound by it.
+inline uint32_t mix_spans(uint32_t cta_chunks, int nr, int dir, bool tweak, uint32_t unit_blocks, bool link) {
+    if (link || unit_blocks < 32 || (tweak && nr == 12)) return 0;
+    const bool big = nr == 14;
+    uint32_t per_span;
+    if (dir == 0) per_span = tweak ? (big ? 1300 : 1400) : (big ? 1200 : 1250);
+    else per_span = tweak ? (big ? 1600 : 1800) : 1300;
+    return cta_chunks / per_span;
+}
+
 constexpr uint32_t kLineBlocks = 8;  // blocks in a 128-byte line
 
 // Lanes that share a page's chain in CBC encryption.  Few pages are a chain's

@@ -3,6 +3,7 @@
 //   "s teams sms"               -> prints cbc_enc_split_ctas
 //   "l sms unit_blocks bytes"   -> prints link_sms
 //   "d sms bpp bytes link"      -> prints cbc_dec_sms
+//   "m cta_chunks nr dir tweak unit_blocks link" -> prints mix_spans
 #include <cstdio>
 
 #include "kgpu_bulk.h"
@@ -32,6 +33,11 @@ int main() {
             unsigned long long bytes;
             if (std::scanf("%d %u %llu %d", &sms, &bpp, &bytes, &link) != 4) return 2;
             std::printf("%d\n", kgpu::cbc_dec_sms(sms, bpp, bytes, link != 0));
+        } else if (kind[0] == 'm') {
+            unsigned chunks, unit;
+            int nr, dir, tweak, link;
+            if (std::scanf("%u %d %d %d %u %d", &chunks, &nr, &dir, &tweak, &unit, &link) != 6) return 2;
+            std::printf("%u\n", kgpu::mix_spans(chunks, nr, dir, tweak != 0, unit, link != 0));
         } else {
             return 2;
         }

@@ -88,3 +88,35 @@ def test_sms_for_cbc_decryption(ask):
     assert ask("d", SMS, 256, 2 * mib, 1) == ask("d", SMS, 32, 48 * mib, 1) == 38
     assert ask("d", SMS, 32, 49 * mib, 1) == ask("d", SMS, 256, 97 * mib, 1) == 114
     assert ask("d", SMS, 16, 64 * mib, 1) == SMS
+
+
+# name in bench.py, name in test_mixed_kernel_gpu.py: rounds, direction, tweak
+MIXED = {("aes256_xts_enc", "ENC256"): (14, 0, 1), ("aes128_xts_enc", "ENC128"): (10, 0, 1),
+         ("aes256_xts_dec", "DEC256"): (14, 1, 1), ("aes128_xts_dec", "DEC128"): (10, 1, 1),
+         ("aes128_ecb_enc", None): (10, 0, 0), ("aes128_cbc_dec", "PLAIN"): (10, 1, 0)}
+
+
+def test_bitsliced_warps_take_part_from_where_the_bench_and_the_tests_say(ask):
+    """The bench scales its lookup bound by the share of the blocks that is
+    looked up, and the tests of the mixed kernels go to their lines: both in
+    chunks a CTA, which the library's rule must agree with."""
+    import bench
+    import test_mixed_kernel_gpu as gpu
+    assert set(bench.CHUNKS_PER_SPAN) == {b for b, _ in MIXED}
+    for (b, g), (nr, dir, tweak) in MIXED.items():
+        line = bench.CHUNKS_PER_SPAN[b]
+        assert g is None or getattr(gpu, g) == line
+        for unit in (32, 256, 1 << 20):
+            assert ask("m", line - 1, nr, dir, tweak, unit, 0) == 0
+            assert ask("m", line, nr, dir, tweak, unit, 0) == 1
+            assert ask("m", 10 * line + 7, nr, dir, tweak, unit, 0) == 10
+        assert ask("m", 10 * line, nr, dir, tweak, 31, 0) == 0      # units under 512 bytes
+        assert ask("m", 10 * line, nr, dir, tweak, 256, 1) == 0     # pages over the link
+    # the spans never exceed what a CTA has: four warps, 32 chunks a span
+    for chunks in (1200, 5000, 13797, 10 ** 6):
+        for nr, dir, tweak in [*MIXED.values(), (12, 0, 0), (12, 1, 0), (14, 0, 0), (14, 1, 0)]:
+            assert 128 * ask("m", chunks, nr, dir, tweak, 256, 0) < chunks
+    assert ask("m", 10 ** 6, 12, 0, 1, 256, 0) == 0                 # there is no XTS-AES-192
+    for nr in (10, 12, 14):                                         # every plain size the GPU tests run
+        for dir in (0, 1):
+            assert ask("m", gpu.PLAIN, nr, dir, 0, 32, 0) >= 1
