@@ -114,7 +114,11 @@ __device__ __forceinline__ void tile_blocks(const ReqDesc& d, uint64_t c0, uint6
         t1 = __shfl_sync(0xffffffffu, z1, srel);
         t2 = __shfl_sync(0xffffffffu, z2, srel);
         t3 = __shfl_sync(0xffffffffu, z3, srel);
-        gf128_mul_xpow(t0, t1, t2, t3, j);
+        const uint4 t = gf128_mul_xpow_call(make_uint4(t0, t1, t2, t3), j);
+        t0 = t.x;
+        t1 = t.y;
+        t2 = t.z;
+        t3 = t.w;
     }
     // the next chunk is fetched while this one is enciphered (one warp runs a
     // tile alone, so the load latency would otherwise add to every step)
@@ -282,7 +286,11 @@ __device__ __forceinline__ void tile_blocks2(const ReqDesc& d, uint64_t c0, uint
         t1 = __shfl_sync(0xffffffffu, z1, srel);
         t2 = __shfl_sync(0xffffffffu, z2, srel);
         t3 = __shfl_sync(0xffffffffu, z3, srel);
-        gf128_mul_xpow(t0, t1, t2, t3, j);
+        const uint4 t = gf128_mul_xpow_call(make_uint4(t0, t1, t2, t3), j);
+        t0 = t.x;
+        t1 = t.y;
+        t2 = t.z;
+        t3 = t.w;
     }
     const uint4 zz = make_uint4(0, 0, 0, 0);
     // the next step's two chunks are fetched while this step's are enciphered

@@ -82,3 +82,26 @@ def test_long_units_cost_no_more_time(ctx, mib):
         assert long < 1.5 * short, (long, short)
     finally:
         ctx.delkey(kh)
+
+
+def test_long_units_served(ctx):
+    import paper_1305_3345_gb300 as kg
+    du, units = (1 << 20) + 16, 3
+    key = w.xts_key(64, 128)
+    data = w.seeded_bytes(64, w.STREAM_DATA, du * units)
+    kh = ctx.setkey(key, True)
+    src = to_dev(data)
+    dst = src.new_empty(src.shape)
+    r = np.zeros(1, dtype=kg.request_dtype())
+    r["mode"], r["key"], r["len"], r["unit_size"], r["dir"] = w.MODE_XTS, kh, du * units, du, 1
+    r["src"], r["dst"], r["sector"] = src.data_ptr(), dst.data_ptr(), 5
+    import torch
+    torch.cuda.synchronize()
+    ctx.serve_start()
+    try:
+        rc, status, _ = ctx.serve_poll(ctx.serve_submit(r))
+        assert rc == 0 and status == 0
+    finally:
+        ctx.serve_stop()
+    assert np.array_equal(to_np(dst), oracle.xts(key, 1, data, du, 5))
+    ctx.delkey(kh)
