@@ -858,8 +858,8 @@ __global__ void __launch_bounds__(kCbcEncStagedThreads, 1) cbc_enc_tma_kernel(co
 //
 // Unit starts are only as aligned as u * du.  Units of a multiple of 8 bytes
 // move in 8-byte accesses; others are read as the two aligned 16-byte words
-// that hold a block and shifted into place, and written in the widest pieces
-// that their address allows.
+// that hold a block and shifted into place, and written as aligned 4-byte words
+// with smaller pieces at their ends.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint4 load_tail_word(const uint8_t* q, const uint8_t* end) {
     // the aligned word at q, of which only the bytes before end are there

@@ -547,10 +547,9 @@ void split_chains(ReqDesc* descs, uint32_t n, const Codes& refused, uint64_t war
 // tile is 32 serial chains of a page's blocks, several times longer, and one
 // handed out last runs alone at the end.  So every CBC-encryption request
 // runs before the tail reserve, the largest other requests holding their
-// last reserve_tiles tiles (two per resident warp: enough short work to keep
-// every warp busy while the long tiles finish); plan_batch, whose kernel keeps a
-// queue for CBC encryption, asks for a reserve of everything.  Ties keep
-// submission order.
+// last reserve_tiles tiles.  plan_batch, the library's one caller, whose kernel
+// keeps a queue for CBC encryption, reserves everything: CBC encryption first,
+// then the rest.  Ties keep submission order.
 // Allocation-free.  Returns the total tile count.
 template <class Codes>
 uint64_t order_batch(const ReqDesc* descs, uint32_t n, const Codes& codes, uint64_t reserve_tiles, uint64_t* prefix,
@@ -602,8 +601,9 @@ uint64_t order_batch(const ReqDesc* descs, uint32_t n, const Codes& codes, uint6
 }
 
 // Fills the header of a batch whose descriptors are packed in buf: lanes per
-// CBC-encryption page, the run order (CBC encryption first, since the kernel keeps a queue of its own for
-// it; smallest first among it and among the rest), the prefix, and how many
+// CBC-encryption page, the run order (CBC encryption first, since the kernel
+// keeps a queue of its own for it; smallest first among it and among the rest),
+// the prefix, and how many
 // warps of a CTA start with CBC encryption: enough that its tiles start
 // together, but no more than a third above its share of the blocks, so that
 // the SMs always have other work beside the chains.  refused(i): request i
